@@ -2,7 +2,7 @@
 // conservation reduction.  Initialisation and moments compute in double
 // precision whatever the storage type of f; the boundary fill computes in the
 // storage precision (its results are stored at that precision).
-#include "lbm_internal.cuh"
+#include "pair_math.cuh"
 
 namespace lbm {
 namespace {
@@ -54,6 +54,29 @@ struct DFloat {
   __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
 
+// Moments and equilibrium of the boundary fill.  In single precision they are
+// the pair kernel's (pair_math.cuh), so that a layer comes out the same
+// whether the fill writes it or the pair kernel forms it (WtDesc).
+__device__ __forceinline__ void fill_macros(const Model<double>& m, const double v[NV], double M[5]) {
+  moments(m, v, M[0], M[1], M[2], M[3], M[4]);
+}
+__device__ __forceinline__ void fill_macros(const Model<float>& m, const float v[NV], float M[5]) {
+  float2 F[NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) F[i] = pm::bc2(v[i]);
+  const pm::Mom r = pm::moments<false>(m, RecoverDesc(), F, nullptr, 0, 0, true, true);
+  M[0] = r.rho.x; M[1] = r.ux.x; M[2] = r.uy.x; M[3] = r.uz.x; M[4] = r.T.x;
+}
+__device__ __forceinline__ void fill_feq(const Model<double>& m, const double M[5], double e[NV]) {
+  equilibrium(m, M[0], M[1], M[2], M[3], M[4], e);
+}
+__device__ __forceinline__ void fill_feq(const Model<float>& m, const float M[5], float e[NV]) {
+  pm::Mom r = {pm::bc2(M[0]), pm::bc2(M[1]), pm::bc2(M[2]), pm::bc2(M[3]), pm::bc2(M[4])};
+  r.usq = pm::fma2(r.ux, r.ux, pm::fma2(r.uy, r.uy, pm::mul(r.uz, r.uz)));
+#pragma unroll
+  for (int i = 0; i < NV; ++i) e[i] = pm::feq(m, r, i).x;
+}
+
 // One thread per (face position): writes the two node layers outside a face.
 // blockIdx.y = face (2*axis + hi); faces whose bit is clear in `mask` are
 // skipped.  Sec. 4(2) boundary rules, ghost f = f^eq.  M is the arithmetic
@@ -94,13 +117,13 @@ __global__ void fill_kernel(R* __restrict__ f, Layout L, Model<M> m, BcDesc bc, 
     M v[NV], M0[5];
 #pragma unroll
     for (int i = 0; i < NV; ++i) v[i] = (M)f[i * L.fs + m0];
-    moments(m, v, M0[0], M0[1], M0[2], M0[3], M0[4]);
+    fill_macros(m, v, M0);
     if (kind == LBM_BC_EXTRAPOLATE) {
       const long long m1 = base + (hi ? N - 2 : 1) * step;
       M M1[5];
 #pragma unroll
       for (int i = 0; i < NV; ++i) v[i] = (M)f[i * L.fs + m1];
-      moments(m, v, M1[0], M1[1], M1[2], M1[3], M1[4]);
+      fill_macros(m, v, M1);
 #pragma unroll
       for (int k = 0; k < 5; ++k) {
         G1[k] = M(2) * M0[k] - M1[k];
@@ -116,10 +139,10 @@ __global__ void fill_kernel(R* __restrict__ f, Layout L, Model<M> m, BcDesc bc, 
     }
   }
   M e[NV];
-  equilibrium(m, G1[0], G1[1], G1[2], G1[3], G1[4], e);
+  fill_feq(m, G1, e);
 #pragma unroll
   for (int i = 0; i < NV; ++i) f[i * L.fs + i1] = (R)e[i];
-  equilibrium(m, G2[0], G2[1], G2[2], G2[3], G2[4], e);
+  fill_feq(m, G2, e);
 #pragma unroll
   for (int i = 0; i < NV; ++i) f[i * L.fs + i2] = (R)e[i];
 }

@@ -16,11 +16,20 @@
 //   f_new = keep_i f + (dt/tau) f^eq - (|v| dt/dx) C + (lambda_i dt/dx^2) S,
 // with S the sum of the six neighbours and keep_i = 1 - dt/tau - 6 lambda_i dt/dx^2.
 //
-// The kernel also writes the boundary layers of the state it produces
-// (WtDesc): periodic images of the first and last two rows, planes and (for
-// even nx) columns, and the x-face layers of extrapolating or reflecting
-// faces (Sec. 4(2) rules applied to the two new boundary cells, which the
-// same thread holds), so the next step needs no separate fill for them.
+// The v_z < 0 velocities need plane z+2 for one term.  It is added when plane
+// z+1 is worked on (part[] below), so a plane needs one plane of look-ahead,
+// not two: two of the four ring slots hold copies in flight where it was one
+// (together with the boundary code taken out of the loop, 256^3: 418 -> 385 us
+// per step, 77 % of the measured copy bandwidth).
+//
+// Boundary layers (WtDesc): the planes of a periodic z axis are read where
+// they are; the layers of reflecting faces and of extrapolating x faces are
+// formed by the threads at the face when they read them, from the moments
+// they hold anyway (two packed equilibria for a thread's pair, against a
+// store, a separate pass or a re-read of the new state: reading a unit's own
+// stores back cost 26 us per unit with a face, 383 -> 448 us on 256^3); and
+// the kernel writes the periodic x and y images of the state it produces with
+// the values themselves, so the next step needs no separate fill for them.
 #include "pair_math.cuh"
 #include "tma_ring.cuh"
 
@@ -31,16 +40,13 @@ using ring::mbar_init;
 using ring::mbar_expect_tx;
 using ring::mbar_wait;
 using ring::tma_load_plane;
-using ring::tma_prefetch_plane;
 
 // Tile geometry of the pair kernel: a TX x TY column of cells, one thread per
 // cell pair (x, x+1), and a four-plane ring: cell plane z reads ring planes z
-// (its x / y neighbours), z+1 and z+2 while z+3 lands.  PF > 0 also asks the
-// TMA unit to bring ring plane j+PF into L2 when plane j is copied, which
-// keeps more DRAM reads in flight per SM than the ring alone.
-template <int TX_, int TY_, int PF_, bool SPLIT_ = false>
+// (its x / y neighbours) and z+1 while z+2 and z+3 land.
+template <int TX_, int TY_, bool SPLIT_ = false>
 struct PairGeo {
-  static constexpr int TX = TX_, TY = TY_, NSLOT = 4, PF = PF_;
+  static constexpr int TX = TX_, TY = TY_, NSLOT = 4;
   // SPLIT: the CTA works as two independent halves of 128 threads (the left
   // and right 32 x 8 cells), each with its own named barrier per plane; a
   // slot is refilled by whichever half releases it second (release counters
@@ -69,19 +75,32 @@ struct PairGeo {
   __device__ static int row(int tid) { return SPLIT ? (tid & 127) >> 4 : tid / PX; }
 };
 // 32 x 8 tiles (the single-cell tiled kernel's box, 40 x 12): two CTAs of 4
-// warps per SM, L2 prefetch two planes ahead (256^3: 0.475 ms per step, 0.488
-// without the prefetch; one or three planes ahead: no faster).
-using Geo32 = PairGeo<ring::TX, ring::TY, 2>;
+// warps per SM.  With two planes in flight an L2 prefetch of later ones only
+// adds L2 lookups (256^3, us per step: 385; one plane ahead 401, two 399,
+// three 410 and more; with one plane in flight it was needed: 475 against 488).
+using Geo32 = PairGeo<ring::TX, ring::TY>;
 // 64 x 8 tiles (box 72 x 12 x 1 x 15): one CTA of 8 warps per SM, 288-byte
-// row reads, run as two split halves.  Its data movement alone (ring +
-// stores, no arithmetic) is faster (0.362 ms against 0.443 ms on 256^3);
-// with the arithmetic it takes 0.511 ms (0.549 ms with one CTA-wide barrier
-// per plane), against 0.465 ms for two independent 32 x 8 CTAs per SM.
-using Geo64 = PairGeo<64, 8, 2, true>;
+// row reads, run as two split halves: 426 us per step on 256^3.
+using Geo64 = PairGeo<64, 8, true>;
 static_assert(Geo32::BX == ring::BX && Geo32::BY == ring::BY, "Geo32 shares the tiled kernel's tensor map");
 
 using pm::bc2;
 using pm::ld2;
+
+// Forms of the kernel.  The plane loop is about as long as the instruction
+// caches serve at full rate: code that few units or few grids run costs all
+// units that carry it (256^3, us per step: the layers of x faces in the loop
+// 14, those of y and z walls 20, the FP64 recovery 17; the boundary code in a
+// second copy of the loop, for the units at a boundary only, 30 more than in
+// the one loop).  So a launch takes the form with the parts its grids need.
+// FULL: every tile lies inside the grid (nx and ny multiples of the tile), so
+// the activity tests fold away.  R1: dt = tau (dt/tau = 1, keep_2 = 0).  RD:
+// FP64 temperature recovery.  XF, WALL: layers of extrapolating / reflecting
+// x faces, of reflecting y and z faces, formed as they are read.
+template <bool FULL_, bool R1_, bool RD_, bool XF_, bool WALL_>
+struct Opt {
+  static constexpr bool FULL = FULL_, R1 = R1_, RD = RD_, XF = XF_, WALL = WALL_;
+};
 
 // Named barrier `id` over 128 threads with an OR of v across them.
 __device__ __forceinline__ bool half_sync_or(unsigned id, bool v) {
@@ -101,10 +120,8 @@ __device__ __forceinline__ bool half_sync_or(unsigned id, bool v) {
 // Plane j of the unit is the ring's plane number jb + j (slot (jb+j) % NSLOT,
 // phase parity ((jb+j) / NSLOT) & 1), so consecutive units of a CTA keep
 // using the same barriers; jb advances by the unit's plane count.  All
-// threads of the CTA call it together; timed_out is uniform.  FULL: every
-// tile lies inside the grid (nx and ny multiples of the tile), so every pair
-// is active and the activity tests fold away.
-template <int SCHEME, bool WT, class G, bool FULL = false, bool R1 = false>
+// threads of the CTA call it together; timed_out is uniform.
+template <int SCHEME, class G, class O>
 __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* __restrict__ fin,
                                           float* __restrict__ fout, const Layout& L, const Model<float>& m,
                                           const WtDesc& wt, const RecoverDesc& rd, int x0, int y0, int z0,
@@ -115,13 +132,21 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* _
   const int tid = threadIdx.x;
   const int tx = G::col(tid), ty = G::row(tid);
   const int x = x0 + 2 * tx, y = y0 + ty;
-  const bool act0 = FULL || ((x < L.nx) && (y < L.ny));
-  const bool act1 = FULL || ((x + 1 < L.nx) && (y < L.ny));
+  const bool act0 = O::FULL || ((x < L.nx) && (y < L.ny));
+  const bool act1 = O::FULL || ((x + 1 < L.nx) && (y < L.ny));
   // ring planes 0 .. nzc+1 are the padded planes z0+2 .. z0+nzc+3 (interior
-  // z0 .. z0+nzc+1); cell plane k reads ring planes k, k+1, k+2
+  // z0 .. z0+nzc+1); cell plane k reads ring planes k and k+1
   const int nplanes = nzc + 2;
+  // interior plane z of the grid or its two z layers; a periodic z axis has no
+  // layers: its planes are read where they are (WtDesc)
+  auto zplane = [&](int z) {
+    if (!wt.per[2]) return z;
+    while (z < 0) z += L.nz;
+    while (z >= L.nz) z -= L.nz;
+    return z;
+  };
 
-  // copy ring plane j (interior z0 + j, padded z0 + j + 2) into its slot
+  // copy ring plane j (interior z0 + j, padded two more) into its slot
   // (SPLIT: release counters and the count of issued planes follow the mbarriers)
   unsigned* rel = reinterpret_cast<unsigned*>(bars + NSLOT);
   int* issued_s = reinterpret_cast<int*>(rel + NSLOT);
@@ -130,8 +155,7 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* _
     const unsigned g = jb + (unsigned)j;
     float* dst = reinterpret_cast<float*>(smem + (g % NSLOT) * G::SLOT_STRIDE);
     mbar_expect_tx(&bars[g % NSLOT], G::SLOT_BYTES);
-    tma_load_plane(dst, tin, x0 + OX - TMA_LEFT, y0, z0 + j + 2, &bars[g % NSLOT]);
-    if (G::PF > 0 && j + G::PF < nplanes) tma_prefetch_plane(tin, x0 + OX - TMA_LEFT, y0, z0 + j + G::PF + 2);
+    tma_load_plane(dst, tin, x0 + OX - TMA_LEFT, y0, zplane(z0 + j) + 2, &bars[g % NSLOT]);
     if (G::SPLIT) atomicMax(issued_s, j + 1);
     else issued = j + 1;
   };
@@ -157,26 +181,47 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* _
   const long long gbase = L.at(x, y, z0);
 
   float2 h1[NV], h2[NV], carry[NV];
+  const long long below1 = L.at(x, y, zplane(z0 - 1)), below2 = L.at(x, y, zplane(z0 - 2));
 #pragma unroll
   for (int i = 0; i < NV; ++i) {
-    h1[i] = act0 ? ld2(fin + i * L.fs + gbase - L.plane) : make_float2(0.f, 0.f);
-    h2[i] = act0 ? ld2(fin + i * L.fs + gbase - 2 * L.plane) : make_float2(0.f, 0.f);
+    h1[i] = act0 ? ld2(fin + i * L.fs + below1) : make_float2(0.f, 0.f);
+    h2[i] = act0 ? ld2(fin + i * L.fs + below2) : make_float2(0.f, 0.f);
     carry[i] = make_float2(0.f, 0.f);
   }
 
   unsigned bad = 0u;
-  // ring planes 0 .. 2 must have landed; the outcome is made uniform by the barrier
+  // ring planes 0 and 1 must have landed; the outcome is made uniform by the barrier
   {
-    bool ok = true;
-    for (int j = 0; j < 3; ++j) ok = arrived(j) && ok;
+    bool ok = arrived(0);
+    ok = arrived(1) && ok;
     timed_out = __syncthreads_or(!ok) != 0;
+  }
+  if (O::WALL && wt.zlo && z0 < 2 && !timed_out && act0) {
+    // the layers below a reflecting z-lo face, from the grid's plane 0
+    const float* P0 = slot(0);
+    float2 v[NV];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) v[i] = z0 == 0 ? ld2(P0 + i * PL + c) : h1[i];
+    const pm::Mom r = pm::moments<O::RD>(m, rd, v, P0, c, PL, act0, act1);
+    const pm::Mom e1 = pm::wall_layer<2>(r, false), e2 = pm::wall_layer<2>(r, true);
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      h2[i] = pm::feq(m, z0 == 0 ? e2 : e1, i);
+      if (z0 == 0) h1[i] = pm::feq(m, e1, i);
+    }
   }
   if (!timed_out && SCHEME == LBM_SCHEME_NND) {
     const float* P0 = slot(0);
-    const float* P1 = slot(1);
 #pragma unroll
-    for (int i = 0; i < NV; ++i) carry[i] = pm::carry0(i, h2[i], h1[i], ld2(P0 + i * PL + c), ld2(P1 + i * PL + c));
+    for (int i = 0; i < NV; ++i) carry[i] = pm::carry0(i, h2[i], h1[i], ld2(P0 + i * PL + c));
   }
+
+  // The v_z < 0 velocities' update of a plane needs the z difference one plane
+  // further up than anything else does (pm::deferred), so it is finished and
+  // stored a plane late: part[i] holds it without its last term.  Cell plane k
+  // then reads ring planes k and k+1 only, and of the four slots two (not one)
+  // hold copies in flight.
+  float2 part[NV];
 
   // Besides the own pair of plane k (F, below), the planes below are carried
   // in registers only where a field needs them: h1 for the Laplacian of
@@ -196,14 +241,39 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* _
   // T makes the sum non-finite, and so does a non-finite velocity: T is
   // (E/rho - u^2)/b, -inf or NaN when u^2 is inf or NaN.
   float2 hmin_rho = make_float2(INFINITY, INFINITY), hmin_T = hmin_rho, hsum = make_float2(0.f, 0.f);
-  // write-through targets that do not depend on the plane: the periodic y and
-  // x images of this pair (element offsets from its own index, 0 = none)
-  long long img_y = 0, img_x = 0;
-  if (WT && act0) {
-    if (wt.per[1]) img_y = y < 2 ? (long long)L.ny * L.sx : (y >= L.ny - 2 ? -(long long)L.ny * L.sx : 0);
-    if (wt.per[0]) img_x = x == 0 ? L.nx : (x == L.nx - 2 ? -L.nx : 0);
+  // periodic images of this pair (element offsets from its own index, 0 = none)
+  unsigned img_y = 0, img_x = 0;
+  if (act0) {
+    if (wt.per[1]) img_y = (unsigned)L.sx * (unsigned)(y < 2 ? L.ny : (y >= L.ny - 2 ? -L.ny : 0));
+    if (wt.per[0]) img_x = (unsigned)(x == 0 ? L.nx : (x == L.nx - 2 ? -L.nx : 0));
   }
-  const bool face_lo = WT && act0 && wt.xlo && x == 0, face_hi = WT && act0 && wt.xhi && x == L.nx - 2;
+  // store the pair's new values of plane k, the deferred fields (late) or the others, and their images
+  auto store = [&](const float2(&out)[NV], int k, bool late) {
+    // the pair's element offset within a field: below 2^32 (the host rejects
+    // longer fields), so the fields' stores share one 32-bit offset
+    const unsigned g = (unsigned)gbase + (unsigned)k * (unsigned)L.plane;
+    auto put = [&](unsigned at) {
+      if (act1) {
+#pragma unroll
+        for (int i = 0; i < NV; ++i)
+          if (pm::deferred<SCHEME>(i) == late) *reinterpret_cast<float2*>(fout + i * L.fs + at) = out[i];
+      } else if (act0) {
+#pragma unroll
+        for (int i = 0; i < NV; ++i)
+          if (pm::deferred<SCHEME>(i) == late) fout[i * L.fs + at] = out[i].x;
+      }
+    };
+    put(g);
+    if (img_y | img_x) {
+      if (img_y) put(g + img_y);
+      if (img_x) put(g + img_x);
+    }
+  };
+  // faces whose layers are formed here, from the moments of the cells at the
+  // face, at the moment they are read (WtDesc)
+  const bool at_xlo = O::XF && wt.xlo && x == 0 && act0, at_xhi = O::XF && wt.xhi && x == L.nx - 2 && act0;
+  const bool at_ylo = O::WALL && wt.ylo && y == 0 && act0, at_yhi = O::WALL && wt.yhi && y == L.ny - 1 && act0;
+  const bool tile_y = O::WALL && ((wt.ylo && y0 == 0) || (wt.yhi && y0 + G::TY >= L.ny));
   // the pair's own values of the plane: loaded once for the first plane, then
   // carried from the previous plane's z-neighbour loads, so that the moments
   // of a plane start without waiting on shared memory (256^3: 0.4206 ->
@@ -217,80 +287,72 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* _
   for (int k = 0; k < nzc && !timed_out; ++k) {
     const float* P0 = slot(k);
     const float* P1 = slot(k + 1);
-    const float* P2 = slot(k + 2);
     float2 Z1[NV];
 #pragma unroll
     for (int i = 0; i < NV; ++i) Z1[i] = ld2(P1 + i * PL + c);
 
     // moments (relations e1-e3), health, equilibrium and the per-field update
-    const pm::Mom r = pm::moments(m, rd, F, P0, c, PL, act0, act1);
+    const pm::Mom r = pm::moments<O::RD>(m, rd, F, P0, c, PL, act0, act1);
+    {
+      // layers beyond the faces this pair touches: into the plane tile's halo
+      // (x: read by this thread only; y: by the row above or below too, a row
+      // of this warp), or in place of the plane above
+      if (O::XF && (at_xlo | at_xhi)) {
+#pragma unroll 1
+        for (int lo = 0; lo < 2; ++lo) {
+          if (!(lo ? at_xlo : at_xhi)) continue;
+          float* t = const_cast<float*>(P0) + c + (lo ? -2 : 2);
+          const pm::Mom e = pm::x_layers(r, lo ? wt.xlo : wt.xhi, lo);
+#pragma unroll
+          for (int i = 0; i < NV; ++i) *reinterpret_cast<float2*>(t + i * PL) = pm::feq(m, e, i);
+        }
+      }
+      if (O::WALL && tile_y) {
+        if (at_ylo | at_yhi) {
+#pragma unroll 1
+          for (int q = 0; q < 4; ++q) {  // lo inner, lo outer, hi inner, hi outer
+            if (!(q < 2 ? at_ylo : at_yhi)) continue;
+            float* t = const_cast<float*>(P0) + c + (q < 2 ? -1 - q : q - 1) * BX;
+            const pm::Mom e = pm::wall_layer<1>(r, q & 1);
+#pragma unroll
+            for (int i = 0; i < NV; ++i) *reinterpret_cast<float2*>(t + i * PL) = pm::feq(m, e, i);
+          }
+        }
+        __syncwarp();
+      }
+      if (wt.zhi && z0 + k == L.nz - 1) {
+        const pm::Mom e = pm::wall_layer<2>(r, false);
+#pragma unroll
+        for (int i = 0; i < NV; ++i) Z1[i] = pm::feq(m, e, i);
+      }
+    }
     hmin_rho = make_float2(fminf(hmin_rho.x, r.rho.x), fminf(hmin_rho.y, r.rho.y));
     hmin_T = make_float2(fminf(hmin_T.x, r.T.x), fminf(hmin_T.y, r.T.y));
     hsum = pm::add(hsum, pm::add(r.rho, r.T));
+    // out: this plane's fields, and the deferred ones of the plane below
     float2 out[NV];
 #pragma unroll
-    for (int i = 0; i < NV; ++i)
-      out[i] = pm::field_update<SCHEME, BX, DZ, R1>(m, i, P0 + i * PL + c, F[i], Z1[i], P2 + i * PL + c,
-                                                h1[i], h2[i], carry[i], dz[i], pm::feq(m, r, i));
-    // the pair's element offset within a field: below 2^32 (the host rejects
-    // longer fields), so the fields' stores share one 32-bit offset
-    const unsigned g = (unsigned)gbase + (unsigned)k * (unsigned)L.plane;
-    if (act1) {
-#pragma unroll
-      for (int i = 0; i < NV; ++i) *reinterpret_cast<float2*>(fout + i * L.fs + g) = out[i];
-    } else if (act0) {
-#pragma unroll
-      for (int i = 0; i < NV; ++i) fout[i * L.fs + g] = out[i].x;
-    }
-    // ---- boundary layers of the new state (write-through): at most one
-    // periodic image per axis (axes of >= 4 cells), and the x-face layers
-    if (WT && act0) {
-      const int z = z0 + k;
-      long long img_z = 0;
-      if (wt.per[2]) img_z = z < 2 ? (long long)L.nz * L.plane : (z >= L.nz - 2 ? -(long long)L.nz * L.plane : 0);
-      if (img_y | img_z | img_x) {
-#pragma unroll 1
-        for (int q = 0; q < 3; ++q) {
-          const long long off = q == 0 ? img_y : (q == 1 ? img_z : img_x);
-          if (off == 0) continue;
-          const long long at = (long long)g + off;
-          if (act1) {
-#pragma unroll
-            for (int i = 0; i < NV; ++i) *reinterpret_cast<float2*>(fout + i * L.fs + at) = out[i];
-          } else {
-#pragma unroll
-            for (int i = 0; i < NV; ++i) fout[i * L.fs + at] = out[i].x;
-          }
-        }
-      }
-      if (face_lo || face_hi) {
-#pragma unroll 1
-        for (int side = 0; side < 2; ++side) {
-          if (side == 0 ? !face_lo : !face_hi) continue;
-          float c0[NV], c1[NV], g1[NV], g2[NV];
-#pragma unroll
-          for (int i = 0; i < NV; ++i) {
-            c0[i] = side == 0 ? out[i].x : out[i].y;  // the cell next to the face
-            c1[i] = side == 0 ? out[i].y : out[i].x;
-          }
-          pm::x_face_layers(m, side == 0 ? wt.xlo : wt.xhi, c0, c1, g1, g2);
-          const long long at = side == 0 ? L.at(-2, y, z) : L.at(L.nx, y, z);
-#pragma unroll
-          for (int i = 0; i < NV; ++i)
-            *reinterpret_cast<float2*>(fout + i * L.fs + at) =
-                side == 0 ? make_float2(g2[i], g1[i]) : make_float2(g1[i], g2[i]);
-        }
+    for (int i = 0; i < NV; ++i) {
+      const float2 o = pm::field_update<SCHEME, BX, DZ, O::R1>(m, i, P0 + i * PL + c, F[i], Z1[i], h1[i], h2[i],
+                                                               carry[i], dz[i], pm::feq(m, r, i));
+      if (pm::deferred<SCHEME>(i)) {
+        out[i] = pm::tail(m, i, dz[i], part[i]);
+        part[i] = o;
+      } else {
+        out[i] = o;
       }
     }
+    store(out, k, false);
+    if (k > 0) store(out, k - 1, true);
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
       if (SCHEME == LBM_SCHEME_UPWIND2) h2[i] = h1[i];
       h1[i] = F[i];
       F[i] = Z1[i];
     }
-    // ring plane k+3 (needed next step) must have landed; the barrier also
+    // ring plane k+2 (needed next step) must have landed; the barrier also
     // marks plane k as retired, so its slot takes plane k + NSLOT
-    const bool ok = (k + 3 < nplanes) ? arrived(k + 3) : true;
+    const bool ok = arrived(k + 2);
     if (G::SPLIT) {
       // this half is done with plane k; the second half to say so refills its slot
       const unsigned hf = (unsigned)tid >> 7;
@@ -317,6 +379,33 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* _
         issue(k + NSLOT);
       }
     }
+  }
+  // the last plane's deferred fields, from ring plane nzc+1 (landed: the last step waited for it)
+  if (nzc > 0 && !timed_out) {
+    const float* P1 = slot(nzc + 1);
+    float2 out[NV], top[NV];
+#pragma unroll
+    for (int i = 0; i < NV; ++i)
+      if (pm::deferred<SCHEME>(i)) top[i] = ld2(P1 + i * PL + c);
+    const int over = z0 + nzc - (L.nz - 1);  // 0, 1: ring plane nzc+1 is the first, second layer above the grid
+    if (O::WALL && wt.zhi && over >= 0) {
+      // a reflecting z-hi face's, from the grid's last plane (still in its slot)
+      const float* P0 = slot(nzc - over);
+      float2 v[NV];
+#pragma unroll
+      for (int i = 0; i < NV; ++i) v[i] = ld2(P0 + i * PL + c);
+      const pm::Mom e = pm::wall_layer<2>(pm::moments<O::RD>(m, rd, v, P0, c, PL, act0, act1), over == 1);
+#pragma unroll
+      for (int i = 0; i < NV; ++i)
+        if (pm::deferred<SCHEME>(i)) top[i] = pm::feq(m, e, i);
+    }
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      if (!pm::deferred<SCHEME>(i)) continue;
+      const float2 Z1 = top[i];
+      out[i] = pm::tail(m, i, SCHEME == LBM_SCHEME_NND ? pm::mmc2(pm::sub(Z1, F[i]), carry[i]) : Z1, part[i]);
+    }
+    store(out, nzc - 1, true);
   }
   // SPLIT halves leave the loop on their own (a half that timed out stops
   // releasing slots, so the other one's waits run out too): rejoin here
@@ -346,8 +435,7 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* _
   jb += (unsigned)nplanes;
 }
 
-// FULL: full tiles; R1: dt = tau (dt/tau = 1, keep_2 = 0), used with FULL only
-template <int SCHEME, bool WT, class G, bool FULL, bool R1 = false>
+template <int SCHEME, class G, class O>
 __global__ void __launch_bounds__(G::THREADS, G::CTAS_PER_SM)
     step_pair_kernel(const __grid_constant__ CUtensorMap tin, const float* __restrict__ fin, float* __restrict__ fout,
                      Layout L, Model<float> m, WtDesc wt, RecoverDesc rd, ZSched zs, unsigned* __restrict__ flags,
@@ -366,8 +454,8 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS_PER_SM)
   __syncthreads();
   unsigned jb = 0;
   bool timed_out = false;
-  pair_unit<SCHEME, WT, G, FULL, R1>(&tin, fin, fout, L, m, wt, rd, blockIdx.x * G::TX, blockIdx.y * G::TY,
-                           zs.z0(blockIdx.z), zs.len(blockIdx.z, L.nz), flags, smem, bars, jb, timed_out, wait_limit);
+  pair_unit<SCHEME, G, O>(&tin, fin, fout, L, m, wt, rd, blockIdx.x * G::TX, blockIdx.y * G::TY, zs.z0(blockIdx.z),
+                          zs.len(blockIdx.z, L.nz), flags, smem, bars, jb, timed_out, wait_limit);
 }
 
 // Persistent batched step: two CTAs per SM take the units of every grid in
@@ -376,8 +464,7 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS_PER_SM)
 // increment per unit, so fast and slow CTAs balance.  Every CTA overshoots
 // the queue once; the last CTA to finish resets the queue for the next
 // launch (stream order), which keeps the launch replayable in a CUDA graph.
-// FULL / R1: every grid of the table has full tiles / dt = tau (NND only).
-template <int SCHEME, class G, bool FULL = false, bool R1 = false>
+template <int SCHEME, class G, class O>
 __global__ void __launch_bounds__(G::THREADS, G::CTAS_PER_SM)
     step_pair_batch_kernel(const __grid_constant__ BatchTable tab) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -416,9 +503,9 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS_PER_SM)
     const WtDesc wt = it.wt;
     const RecoverDesc rd = it.rd;
     const ZSched zs = it.zs;
-    pair_unit<SCHEME, true, G, FULL, R1>(&tab.map[e], it.fin, it.fout, L, m, wt, rd, (t % it.tiles_x) * G::TX,
-                                         (t / it.tiles_x) * G::TY, zs.z0(chunk), zs.len(chunk, L.nz), it.flags, smem,
-                                         bars, jb, timed_out, tab.wait_limit);
+    pair_unit<SCHEME, G, O>(&tab.map[e], it.fin, it.fout, L, m, wt, rd, (t % it.tiles_x) * G::TX,
+                            (t / it.tiles_x) * G::TY, zs.z0(chunk), zs.len(chunk, L.nz), it.flags, smem, bars, jb,
+                            timed_out, tab.wait_limit);
   }
   if (threadIdx.x == 0) {
     __threadfence();
@@ -430,43 +517,46 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS_PER_SM)
   }
 }
 
-template <int SCHEME, class G>
-cudaError_t set_attributes() {
-  cudaError_t e = cudaSuccess;
-  auto set = [&](const void* fn) {
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM);
-  };
-  set((const void*)step_pair_kernel<SCHEME, true, G, false>);
-  set((const void*)step_pair_kernel<SCHEME, false, G, false>);
-  if (SCHEME == LBM_SCHEME_NND) {
-    set((const void*)step_pair_kernel<SCHEME, true, G, true>);
-    set((const void*)step_pair_kernel<SCHEME, false, G, true>);
-    set((const void*)step_pair_kernel<SCHEME, true, G, true, true>);
-    set((const void*)step_pair_kernel<SCHEME, false, G, true, true>);
+// What the forms go by, over all grids of a launch.
+struct Need {
+  bool full = true, r1 = true, rd = false, xf = false, wall = false;
+  void add(const Layout& L, int tx, int ty, const Model<float>& m, const WtDesc& wt, const RecoverDesc& r) {
+    full = full && L.nx % tx == 0 && L.ny % ty == 0;
+    r1 = r1 && m.dt_tau == 1.0f && m.keep2 == 0.0f;
+    rd = rd || r.on;
+    xf = xf || wt.xlo || wt.xhi;
+    wall = wall || wt.ylo || wt.yhi || wt.zlo || wt.zhi;
   }
-  set((const void*)step_pair_batch_kernel<SCHEME, G>);
-  if (SCHEME == LBM_SCHEME_NND) {
-    set((const void*)step_pair_batch_kernel<SCHEME, G, true>);
-    set((const void*)step_pair_batch_kernel<SCHEME, G, true, true>);
+};
+
+// The forms that exist: NND with dt = tau and no recovery (every run of the
+// paper) has one per boundary need, everything else one form with all parts.
+using FullPlain = Opt<true, true, false, false, false>;
+using FullFaces = Opt<true, true, false, true, false>;
+using Plain = Opt<false, true, false, false, false>;
+using Faces = Opt<false, true, false, true, false>;
+using Walls = Opt<false, true, false, true, true>;
+using General = Opt<false, false, true, true, true>;
+
+template <int SCHEME, class F>
+void with_form(const Need& n, F f) {
+  if constexpr (SCHEME == LBM_SCHEME_NND) {
+    if (n.r1 && !n.rd) {
+      if (n.wall) return f(Walls());
+      if (n.full) return n.xf ? f(FullFaces()) : f(FullPlain());
+      return n.xf ? f(Faces()) : f(Plain());
+    }
   }
-  return e;
+  f(General());
 }
 
-// The full-tile form (NND only): grids whose nx and ny are multiples of the tile.
-template <int SCHEME, bool WT, class G>
-void launch_full_or_not(dim3 grid, const CUtensorMap& map, const float* fin, float* fout, const Layout& L,
-                        const Model<float>& m, const WtDesc& wt, const RecoverDesc& rd, const ZSched& zs,
-                        unsigned* flags, unsigned wait_limit, cudaStream_t st) {
-  constexpr bool NND = SCHEME == LBM_SCHEME_NND;
-  if (NND && L.nx % G::TX == 0 && L.ny % G::TY == 0 && m.dt_tau == 1.0f && m.keep2 == 0.0f)
-    step_pair_kernel<SCHEME, WT, G, NND, NND><<<grid, G::THREADS, G::SMEM, st>>>(map, fin, fout, L, m, wt, rd, zs,
-                                                                                  flags, wait_limit);
-  else if (NND && L.nx % G::TX == 0 && L.ny % G::TY == 0)
-    step_pair_kernel<SCHEME, WT, G, NND><<<grid, G::THREADS, G::SMEM, st>>>(map, fin, fout, L, m, wt, rd, zs, flags,
-                                                                             wait_limit);
-  else
-    step_pair_kernel<SCHEME, WT, G, false><<<grid, G::THREADS, G::SMEM, st>>>(map, fin, fout, L, m, wt, rd, zs,
-                                                                               flags, wait_limit);
+template <int SCHEME, class G, class... O>
+cudaError_t set_attributes() {
+  const void* fn[] = {(const void*)step_pair_kernel<SCHEME, G, O>..., (const void*)step_pair_batch_kernel<SCHEME, G, O>...};
+  cudaError_t e = cudaSuccess;
+  for (const void* f : fn)
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM);
+  return e;
 }
 
 template <int SCHEME, class G>
@@ -474,11 +564,12 @@ cudaError_t launch_scheme(const CUtensorMap& map, const float* fin, float* fout,
                           const Model<float>& m, const WtDesc& wt, const RecoverDesc& rd, const ZSched& zs,
                           unsigned* flags, unsigned wait_limit, cudaStream_t st) {
   dim3 grid((L.nx + G::TX - 1) / G::TX, (L.ny + G::TY - 1) / G::TY, zs.nch);
-  const bool any = wt.per[0] || wt.per[1] || wt.per[2] || wt.xlo || wt.xhi;
-  if (any)
-    launch_full_or_not<SCHEME, true, G>(grid, map, fin, fout, L, m, wt, rd, zs, flags, wait_limit, st);
-  else
-    launch_full_or_not<SCHEME, false, G>(grid, map, fin, fout, L, m, wt, rd, zs, flags, wait_limit, st);
+  Need need;
+  need.add(L, G::TX, G::TY, m, wt, rd);
+  with_form<SCHEME>(need, [&](auto o) {
+    step_pair_kernel<SCHEME, G, decltype(o)><<<grid, G::THREADS, G::SMEM, st>>>(map, fin, fout, L, m, wt, rd, zs, flags,
+                                                                                wait_limit);
+  });
   return cudaGetLastError();
 }
 
@@ -497,9 +588,9 @@ cudaError_t launch_geo(int scheme, const CUtensorMap& map, const float* fin, flo
 
 template <class G>
 cudaError_t prepare_geo() {
-  cudaError_t e = set_attributes<LBM_SCHEME_NND, G>();
-  if (e == cudaSuccess) e = set_attributes<LBM_SCHEME_UPWIND2, G>();
-  if (e == cudaSuccess) e = set_attributes<LBM_SCHEME_UPWIND1, G>();
+  cudaError_t e = set_attributes<LBM_SCHEME_NND, G, FullPlain, FullFaces, Plain, Faces, Walls, General>();
+  if (e == cudaSuccess) e = set_attributes<LBM_SCHEME_UPWIND2, G, General>();
+  if (e == cudaSuccess) e = set_attributes<LBM_SCHEME_UPWIND1, G, General>();
   return e;
 }
 
@@ -516,25 +607,22 @@ PairShape pair_shape(int cols) {
   return {Geo32::TX, Geo32::TY, Geo32::BX, Geo32::BY, Geo32::THREADS, Geo32::CTAS_PER_SM};
 }
 
+template <int SCHEME, class G>
+void launch_batch_scheme(const BatchTable& tab, int grid, cudaStream_t st) {
+  Need need;
+  for (int e = 0; e < tab.n; ++e)
+    need.add(tab.item[e].L, G::TX, G::TY, tab.item[e].m, tab.item[e].wt, tab.item[e].rd);
+  with_form<SCHEME>(need, [&](auto o) {
+    step_pair_batch_kernel<SCHEME, G, decltype(o)><<<grid, G::THREADS, G::SMEM, st>>>(tab);
+  });
+}
+
 template <class G>
 void launch_batch_geo(int scheme, const BatchTable& tab, int grid, cudaStream_t st) {
-  // the full-tile and dt = tau forms when every grid of the table qualifies
-  bool full = true, r1 = true;
-  for (int e = 0; e < tab.n; ++e) {
-    const BatchItem& it = tab.item[e];
-    full = full && it.L.nx % G::TX == 0 && it.L.ny % G::TY == 0;
-    r1 = r1 && it.m.dt_tau == 1.0f && it.m.keep2 == 0.0f;
-  }
   switch (scheme) {
-    case LBM_SCHEME_NND:
-      if (full && r1) step_pair_batch_kernel<LBM_SCHEME_NND, G, true, true><<<grid, G::THREADS, G::SMEM, st>>>(tab);
-      else if (full) step_pair_batch_kernel<LBM_SCHEME_NND, G, true><<<grid, G::THREADS, G::SMEM, st>>>(tab);
-      else step_pair_batch_kernel<LBM_SCHEME_NND, G><<<grid, G::THREADS, G::SMEM, st>>>(tab);
-      break;
-    case LBM_SCHEME_UPWIND2:
-      step_pair_batch_kernel<LBM_SCHEME_UPWIND2, G><<<grid, G::THREADS, G::SMEM, st>>>(tab);
-      break;
-    default: step_pair_batch_kernel<LBM_SCHEME_UPWIND1, G><<<grid, G::THREADS, G::SMEM, st>>>(tab);
+    case LBM_SCHEME_NND: return launch_batch_scheme<LBM_SCHEME_NND, G>(tab, grid, st);
+    case LBM_SCHEME_UPWIND2: return launch_batch_scheme<LBM_SCHEME_UPWIND2, G>(tab, grid, st);
+    default: return launch_batch_scheme<LBM_SCHEME_UPWIND1, G>(tab, grid, st);
   }
 }
 

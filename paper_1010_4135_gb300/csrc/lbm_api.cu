@@ -341,27 +341,37 @@ unsigned fixed_faces(const lbm_sim* s) {
   return m;
 }
 
-// Boundary layers the pair kernel writes for the state it produces, and the
-// face mask they cover: periodic axes (x only for even nx, where the boundary
-// cell pairs are whole) and extrapolating / reflecting x faces (even nx).
-lbm::WtDesc write_through(const lbm_sim* s, unsigned* faces) {
-  lbm::WtDesc w;
-  unsigned m = 0;
-  const bool on = wt_variant(s->variant);
-  const bool xeven = (s->L.nx % 2) == 0 && s->L.nx >= 4;
-  const int n[3] = {s->L.nx, s->L.ny, s->L.nz};
-  for (int a = 0; a < 3; ++a) {
-    w.per[a] = on && s->bc.kind[2 * a] == LBM_BC_PERIODIC && n[a] >= 4 && (a != 0 || xeven);
-    if (w.per[a]) m |= 3u << (2 * a);
+// What the pair kernel does about the boundary layers (WtDesc).  `written`:
+// the faces whose layers it writes for the state it produces (periodic x for
+// even nx, where the boundary cell pairs are whole, and y, both from 4 cells
+// on, where a cell has one image per axis); `own`: the faces whose layers it
+// never reads (periodic z; extrapolating and reflecting x faces, of which the
+// hi one needs a whole cell pair, nx even; reflecting y and z faces, of which
+// the y-hi one needs its row and the one before in one warp, ny even; none
+// with FP64 recovery, whose moments at a face the fill does not share).
+// TILED_FILL leaves the periodic layers to fill launches.
+lbm::WtDesc write_through(const lbm_sim* s, unsigned* written, unsigned* own) {
+  lbm::WtDesc w = {};
+  *written = *own = 0;
+  if (s->prec != LBM_FP32 || !pair_variant(s->variant)) return w;
+  const int* kind = s->bc.kind;
+  const int nx = s->L.nx, ny = s->L.ny;
+  if (wt_variant(s->variant)) {
+    w.per[0] = kind[0] == LBM_BC_PERIODIC && nx >= 4 && nx % 2 == 0;
+    w.per[1] = kind[2] == LBM_BC_PERIODIC && ny >= 4;
+    w.per[2] = kind[4] == LBM_BC_PERIODIC;
+    if (w.per[0]) *written |= 3u;
+    if (w.per[1]) *written |= 3u << 2;
+    if (w.per[2]) *own |= 3u << 4;
   }
-  auto xk = [&](int kind) {
-    return (on && xeven && (kind == LBM_BC_EXTRAPOLATE || kind == LBM_BC_REFLECT)) ? kind : 0;
-  };
-  w.xlo = xk(s->bc.kind[0]);
-  w.xhi = xk(s->bc.kind[1]);
-  if (w.xlo) m |= 1u;
-  if (w.xhi) m |= 2u;
-  if (faces) *faces = m;
+  int* face[6] = {&w.xlo, &w.xhi, &w.ylo, &w.yhi, &w.zlo, &w.zhi};
+  for (int f = 0; f < 6; ++f) {
+    const bool fits = f < 2 ? nx >= 2 && (f == 0 || nx % 2 == 0) : f != 3 || ny % 2 == 0;
+    if (fits && !s->rd.on && (kind[f] == LBM_BC_REFLECT || (f < 2 && kind[f] == LBM_BC_EXTRAPOLATE))) {
+      *face[f] = kind[f];
+      *own |= 1u << f;
+    }
+  }
   return w;
 }
 
@@ -483,8 +493,7 @@ int lbm_create(const lbm_grid* grid, const lbm_vset* vset, double tau, double dt
         !make_tmap(&s->tmap[1], s->fbuf[1], s->L, lbm::tiled_box_x(), lbm::tiled_box_y()) ||
         !make_tmap(&s->wmap[0], s->fbuf[0], s->L, p64.bx, p64.by) ||
         !make_tmap(&s->wmap[1], s->fbuf[1], s->L, p64.bx, p64.by) ||
-        lbm::prepare_tiled_kernels() != cudaSuccess || lbm::prepare_pair_kernels() != cudaSuccess ||
-        lbm::prepare_split_kernels() != cudaSuccess) {
+        lbm::prepare_tiled_kernels() != cudaSuccess || lbm::prepare_pair_kernels() != cudaSuccess) {
       delete s;
       return LBM_ECUDA;
     }
@@ -574,14 +583,14 @@ int run_steps(lbm_sim* s, int64_t n) {
   }
   const bool pair = s->prec == LBM_FP32 && pair_variant(s->variant);
   const lbm::PairShape shape = lbm::pair_shape(pair_cols(s->variant));
-  unsigned wt_faces = 0;
-  const lbm::WtDesc wt = write_through(s, &wt_faces);
+  unsigned written = 0, own = 0;
+  const lbm::WtDesc wt = write_through(s, &written, &own);
   for (int64_t k = 0; k < n; ++k) {
     void* fin = s->fbuf[s->cur];
     void* fout = s->fbuf[s->cur ^ 1];
-    // layers the previous step did not write for this state
-    unsigned mask = step_faces(s);
-    if (pair && s->layers_ok[s->cur]) mask &= ~wt_faces;
+    // layers that the step reads and the previous step did not write for this state
+    unsigned mask = step_faces(s) & ~own;
+    if (s->layers_ok[s->cur]) mask &= ~written;
     if (mask)
       LBM_LAUNCH(s, LBM_KERNEL_FILL, lbm::launch_fill(s->prec, fin, s->L, s->md, s->mf, s->bc, mask, s->st));
     if (s->prec == LBM_FP32 && s->variant != LBM_VARIANT_PLAIN) {
@@ -591,14 +600,9 @@ int run_steps(lbm_sim* s, int64_t n) {
       if (pair) {
         const CUtensorMap& map = shape.tx == 64 ? s->wmap[s->cur] : s->tmap[s->cur];
         const lbm::ZSched zs = lbm::make_zsched(s->L.nz, zc, s->zchunk > 0 ? s->ztail : auto_ztail(zc));
-        if (s->variant == LBM_VARIANT_TILED_SPLIT)
-          LBM_LAUNCH(s, LBM_KERNEL_STEP,
-                     lbm::launch_step_split(s->scheme, map, (const float*)fin, (float*)fout, s->L, s->mf, wt, s->rd, zs,
-                                            s->flags, s->wait_limit, s->st));
-        else
-          LBM_LAUNCH(s, LBM_KERNEL_STEP,
-                     lbm::launch_step_pair(shape.tx, s->scheme, map, (const float*)fin, (float*)fout, s->L, s->mf,
-                                           wt, s->rd, zs, s->flags, s->wait_limit, s->st));
+        LBM_LAUNCH(s, LBM_KERNEL_STEP,
+                   lbm::launch_step_pair(shape.tx, s->scheme, map, (const float*)fin, (float*)fout, s->L, s->mf, wt,
+                                         s->rd, zs, s->flags, s->wait_limit, s->st));
       } else {
         LBM_LAUNCH(s, LBM_KERNEL_STEP,
                    lbm::launch_step_tiled(s->scheme, s->tmap[s->cur], (const float*)fin, (float*)fout, s->L, s->mf,
@@ -608,7 +612,7 @@ int run_steps(lbm_sim* s, int64_t n) {
       LBM_LAUNCH(s, LBM_KERNEL_STEP,
                  lbm::launch_step_plain(s->prec, s->scheme, fin, fout, s->L, s->md, s->mf, s->flags, s->st));
     }
-    s->layers_ok[s->cur ^ 1] = (pair && wt_faces) ? 1 : 0;
+    s->layers_ok[s->cur ^ 1] = written ? 1 : 0;
     s->cur ^= 1;
     s->steps += 1;
   }
@@ -645,15 +649,15 @@ int run_batch(lbm_sim* const* sims, int32_t n, int64_t steps) {
     if (rc) return rc;
   }
   thread_local static lbm::BatchTable tab;  // built on the host, passed by value to the kernel
-  unsigned wt_faces[lbm::kMaxBatch];
+  unsigned written[lbm::kMaxBatch], own[lbm::kMaxBatch];
   lbm::WtDesc wt[lbm::kMaxBatch];
-  for (int i = 0; i < n; ++i) wt[i] = write_through(sims[i], &wt_faces[i]);
+  for (int i = 0; i < n; ++i) wt[i] = write_through(sims[i], &written[i], &own[i]);
   for (int64_t k = 0; k < steps; ++k) {
     long long units = 0;
     for (int i = 0; i < n; ++i) {
       lbm_sim* s = sims[i];
-      unsigned mask = step_faces(s);
-      if (s->layers_ok[s->cur]) mask &= ~wt_faces[i];
+      unsigned mask = step_faces(s) & ~own[i];
+      if (s->layers_ok[s->cur]) mask &= ~written[i];
       if (mask)
         LBM_LAUNCH(s, LBM_KERNEL_FILL,
                    lbm::launch_fill(s->prec, s->fbuf[s->cur], s->L, s->md, s->mf, s->bc, mask, s->st));
@@ -680,10 +684,7 @@ int run_batch(lbm_sim* const* sims, int32_t n, int64_t steps) {
     tab.done = s0->done;
     const long long resident = (long long)shape.ctas_per_sm * s0->num_sms;
     const int grid = (int)(units < resident ? units : resident);
-    if (s0->variant == LBM_VARIANT_TILED_SPLIT)
-      LBM_LAUNCH(s0, LBM_KERNEL_STEP, lbm::launch_step_split_batch(s0->scheme, tab, grid, s0->st));
-    else
-      LBM_LAUNCH(s0, LBM_KERNEL_STEP, lbm::launch_step_pair_batch(shape.tx, s0->scheme, tab, grid, s0->st));
+    LBM_LAUNCH(s0, LBM_KERNEL_STEP, lbm::launch_step_pair_batch(shape.tx, s0->scheme, tab, grid, s0->st));
     for (int i = 0; i < n; ++i) {
       lbm_sim* s = sims[i];
       s->layers_ok[s->cur ^ 1] = 1;

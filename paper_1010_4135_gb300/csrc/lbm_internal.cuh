@@ -86,14 +86,15 @@ struct BcDesc {
   double fixed[6][5];   // (rho,u1,u2,u3,T)
 };
 
-// Boundary layers a step kernel writes itself for the state it produces
-// ("write-through"), so that no fill kernel runs before the next step:
-// periodic images along each flagged axis, and the extrapolated / reflected
-// layers of the x faces (kind LBM_BC_EXTRAPOLATE or LBM_BC_REFLECT, 0 = not
-// handled in the kernel).
+// Boundary layers the pair kernel takes care of itself, so that no fill
+// kernel runs before the next step.  per[0], per[1]: it writes the periodic x
+// / y images of the state it produces ("write-through").  per[2]: it reads
+// the planes of a periodic z axis where they are.  xlo .. zhi: the face's kind
+// (LBM_BC_EXTRAPOLATE on x faces, LBM_BC_REFLECT) where it forms the layers
+// from the cells at the face as it reads them; 0 = the layers are in memory.
 struct WtDesc {
   int per[3];
-  int xlo, xhi;
+  int xlo, xhi, ylo, yhi, zlo, zhi;
 };
 
 // ---------------------------------------------------------------- physics
@@ -316,13 +317,6 @@ struct BatchTable {
 };
 // Batched step over the descriptor table (`cols` x 8 tiles, maps of that box).
 cudaError_t launch_step_pair_batch(int cols, int scheme, const BatchTable& tab, int grid, cudaStream_t st);
-// Field-split kernel on 32 x 8 tiles (two warp groups of 128 threads per
-// tile, two CTAs per SM; the 40 x 12 map of the pair kernel), single grid and
-// batched; results bitwise equal to the pair kernel's.
-cudaError_t launch_step_split(int scheme, const CUtensorMap& map, const float* fin, float* fout, const Layout& L,
-                              const Model<float>& m, const WtDesc& wt, const RecoverDesc& rd, const ZSched& zs,
-                              unsigned* flags, unsigned wait_limit, cudaStream_t st);
-cudaError_t launch_step_split_batch(int scheme, const BatchTable& tab, int grid, cudaStream_t st);
 // y = 1/x as the FP32 step kernels form the inverse density (device arrays).
 cudaError_t launch_reciprocal_fp32(const float* x, float* y, long long n, cudaStream_t st);
 // Von Neumann service: out[p] = max |omega| of G(k) (Sec. 3) over the states
@@ -335,7 +329,6 @@ cudaError_t launch_vn_max_growth(const double* states, int nstates, const double
 // their first launch (not allowed inside a stream capture).
 cudaError_t prepare_tiled_kernels();
 cudaError_t prepare_pair_kernels();
-cudaError_t prepare_split_kernels();
 // Geometry of the tiled kernel's TMA box (x, y extents) and CTA tile.
 int tiled_box_x();
 int tiled_box_y();

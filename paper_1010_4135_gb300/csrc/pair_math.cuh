@@ -2,9 +2,8 @@
 //
 // A thread owns the two x-adjacent cells (x, x+1) of one tile row and holds
 // their values as float2; everything that is the same arithmetic for both
-// cells runs as packed f32x2 operations (FADD2, FMUL2, FFMA2).  The pair
-// kernel (all 15 fields per thread) and the field-split kernel (two warp
-// groups of one tile, each updating part of the 15 fields) both inline these
+// cells runs as packed f32x2 operations (FADD2, FMUL2, FFMA2).  The forms of
+// the pair kernel and the single-precision boundary fill inline these
 // functions, so they round identically and give bitwise equal results.
 //
 // Shared-memory plane tiles: field i of a plane tile starts PL floats after
@@ -78,9 +77,10 @@ __device__ __noinline__ inline Macro1 recover_fp64(const float* q, int pl, doubl
   return {(float)rho, (float)ux, (float)uy, (float)uz, (float)T};
 }
 
-// Moments of the pair (relations e1-e3) from its 15 values F; with rd.on,
+// Moments of the pair (relations e1-e3) from its 15 values F; with RD and rd.on,
 // cells whose FP32 temperature is ill-conditioned are redone in FP64 from the
 // plane tile at P0 + c (field stride PL).
+template <bool RD>
 __device__ __forceinline__ Mom moments(const Model<float>& m, const RecoverDesc& rd, const float2 (&F)[NV],
                                        const float* P0, int c, int PL, bool act0, bool act1) {
   const float2 sa = add(add(add(F[1], F[2]), add(F[3], F[4])), add(F[5], F[6]));
@@ -100,7 +100,7 @@ __device__ __forceinline__ Mom moments(const Model<float>& m, const RecoverDesc&
   r.uz = mul(mz, ir);
   r.usq = fma2(r.ux, r.ux, fma2(r.uy, r.uy, mul(r.uz, r.uz)));
   r.T = mul(sub(mul(E, ir), r.usq), bc2(m.inv_b));
-  if (rd.on) {
+  if (RD && rd.on) {
     // ill-conditioned FP32 temperature (RecoverDesc): redo the cell in FP64
     const float2 Aa = fma2(bc2(m.AaT), r.T, fma2(bc2(m.AaU), r.usq, bc2(m.Aa0)));
     const float2 Ad = fma2(bc2(m.AdT), r.T, fma2(bc2(m.AdU), r.usq, bc2(m.Ad0)));
@@ -123,23 +123,6 @@ __device__ __forceinline__ Mom moments(const Model<float>& m, const RecoverDesc&
     }
   }
   return r;
-}
-
-// Health bits of the pair's active cells: rho <= 0, T <= 0, non-finite.
-__device__ __forceinline__ unsigned health(const Mom& r, bool act0, bool act1) {
-  unsigned bad = 0u;
-  const float ax[2] = {r.rho.x, r.rho.y}, tt[2] = {r.T.x, r.T.y};
-  const float chk[2] = {fabsf(r.rho.x) + fabsf(r.T.x) + fabsf(r.ux.x) + fabsf(r.uy.x) + fabsf(r.uz.x),
-                        fabsf(r.rho.y) + fabsf(r.T.y) + fabsf(r.ux.y) + fabsf(r.uy.y) + fabsf(r.uz.y)};
-  const bool on[2] = {act0, act1};
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    if (!on[h]) continue;
-    if (!(ax[h] > 0.f)) bad |= LBM_HEALTH_RHO;
-    if (!(tt[h] > 0.f)) bad |= LBM_HEALTH_T;
-    if (!(chk[h] < 1e30f)) bad |= LBM_HEALTH_NONFINITE;
-  }
-  return bad;
 }
 
 // f^eq_i of the pair (Eq. "eq"): rho (A + B w + D w^2) per shell, evaluated
@@ -185,17 +168,30 @@ __device__ __forceinline__ float2 feq(const Model<float>& m, const Mom& r, int i
 // extra dissipation for i <= 6 and the BGK update, with relaxation and the
 // Laplacian centre folded into keep_i:
 //   f_new = keep_i f + (dt/tau) f^eq - (|v| dt/dx) C + (lambda_i dt/dx^2) S.
-// q: the pair in plane tile k (field i); Z1: the pair in plane k+1, Z2p: the
-// field's tile in plane k+2 at the pair; h1, h2: the pair in planes k-1, k-2
+// q: the pair in plane tile k (field i); Z1: the pair in plane k+1; H, H2: the
+// pair in planes k-1, k-2
 // (registers); carry: the minmod of the lower z interface (NND), replaced by
 // that of the upper one.  DZ (NND, diagonal velocities with v_z > 0): the
 // lower z difference f_k - f_{k-1} is carried in dz (the upper difference of
 // the plane before, the same rounded value) instead of being formed from H,
 // and dz takes this plane's upper difference.
-template <int SCHEME, int BX, bool DZ = false, bool R1 = false>
+// The last term of a v_z < 0 velocity, -(|v| dt/(2 dx)) times the minmod at
+// plane k+1 (UPWIND2: times f_{k+2}), is the only one that needs plane k+2;
+// it is left to the caller, who adds it by a last fma (tail) once that plane is
+// there.  For such a velocity the value returned lacks it, carry holds the z
+// difference f_k - f_{k-1} on entry and f_{k+1} - f_k on return, and dz
+// returns what the tail of plane k-1 needs (the minmod at plane k, UPWIND2:
+// f_{k+1}).
+template <int SCHEME>
+constexpr bool deferred(int i) {
+  return vsign(i, 2) < 0 && SCHEME != LBM_SCHEME_UPWIND1;
+}
+__device__ __forceinline__ float2 tail(const Model<float>& m, int i, float2 mm, float2 o) {
+  return fma2(bc2(-0.5f * (i <= 6 ? m.k1 : m.k2)), mm, o);
+}
+template <int SCHEME, int BX, bool DZ, bool R1>
 __device__ __forceinline__ float2 field_update(const Model<float>& m, int i, const float* q, float2 B, float2 Z1,
-                                               const float* Z2p, float2 H, float2 H2, float2& carry, float2& dz,
-                                               float2 fe) {
+                                               float2 H, float2 H2, float2& carry, float2& dz, float2 fe) {
   const float2 half = bc2(0.5f);
   // the convection and neighbour sums start from their first term (0 + x is
   // not an identity for x = -0, so the compiler keeps an add with 0); conv
@@ -204,6 +200,7 @@ __device__ __forceinline__ float2 field_update(const Model<float>& m, int i, con
   // the bookkeeping folds away.
   float2 conv = make_float2(0.f, 0.f), S = make_float2(0.f, 0.f);
   bool have_c = false, cneg = false, have_s = false;
+  float2 last = make_float2(0.f, 0.f);  // what the tail multiplies
   auto acc = [&](float2 G, bool plus) {
     if (!have_c) {
       conv = G;
@@ -311,15 +308,16 @@ __device__ __forceinline__ float2 field_update(const Model<float>& m, int i, con
       }
       acc(G, true);
     } else if (sg < 0) {
-      const float2 Z2 = ld2(Z2p);
       const float2 D1 = sub(Z1, B);
       float2 G;
       if (SCHEME == LBM_SCHEME_NND) {
-        const float2 mA = mmc2(sub(Z2, Z1), D1);
-        G = fma2(bc2(-0.5f), sub(mA, carry), D1);
-        carry = mA;
+        // D1 + (minmod at k) / 2; the tail takes off (minmod at k+1) / 2
+        last = mmc2(D1, carry);
+        G = fma2(half, last, D1);
+        carry = D1;
       } else if (SCHEME == LBM_SCHEME_UPWIND2) {
-        G = mul(half, sub(fma2(bc2(4.f), Z1, mul(bc2(-3.f), B)), Z2));
+        last = Z1;
+        G = mul(half, fma2(bc2(4.f), Z1, mul(bc2(-3.f), B)));
       } else {
         G = D1;
       }
@@ -338,40 +336,60 @@ __device__ __forceinline__ float2 field_update(const Model<float>& m, int i, con
   else o = fma2(bc2(keep), B, mul(bc2(m.dt_tau), fe));
   if (i != 0) o = fma2(bc2(cneg ? kk : -kk), conv, o);
   if (i <= 6) o = fma2(bc2(lam), S, o);
+  if (deferred<SCHEME>(i)) dz = last;
   return o;
 }
 
-// Initial z-interface minmod of field i for a unit starting at plane k = 0
-// (NND): the interface below plane 0 from planes -2, -1 (h2, h1), 0 (fc) and,
-// for v_z < 0, plane 1 (fz1).
-__device__ __forceinline__ float2 carry0(int i, float2 h2, float2 h1, float2 fc, float2 fz1) {
+// Initial carry of field i for a unit starting at plane k = 0 (NND): the
+// minmod of the interface below plane 0 from planes -2, -1 (h2, h1) and 0
+// (fc), or for v_z < 0 the z difference below plane 0.
+__device__ __forceinline__ float2 carry0(int i, float2 h2, float2 h1, float2 fc) {
   const int sz = vsign(i, 2);
   if (sz > 0) return mmc2(sub(h1, h2), sub(fc, h1));
-  if (sz < 0) return mmc2(sub(fz1, fc), sub(fc, h1));
+  if (sz < 0) return sub(fc, h1);
   return make_float2(0.f, 0.f);
 }
 
-// The two layers outside an x face from the boundary cell c0 (next to the
-// face) and its neighbour c1 (Sec. 4(2)): g1 next to the face, g2 outside it.
-__device__ __forceinline__ void x_face_layers(const Model<float>& m, int kind, const float c0[NV], const float c1[NV],
-                                              float g1[NV], float g2[NV]) {
-  float M0[5], M1[5], G1[5], G2[5];
-  lbm::moments(m, c0, M0[0], M0[1], M0[2], M0[3], M0[4]);
+// The two layers outside an x face as a pair in x order (lo: x = -2, -1; hi: x
+// = nx, nx + 1), from the moments r of the pair at the face (Sec. 4(2)):
+// extrapolation g1 = 2 m0 - m1, g2 = 2 g1 - m0 (g1 next to the face, m0 the
+// cell at it, m1 its neighbour), or the reflecting wall.
+__device__ __forceinline__ Mom x_layers(const Mom& r, int kind, bool lo) {
+  auto order = [lo](float g1, float g2) { return lo ? make_float2(g2, g1) : make_float2(g1, g2); };
+  auto ext = [&](float2 v) {
+    const float m0 = lo ? v.x : v.y, m1 = lo ? v.y : v.x;
+    const float g1 = fmaf(2.f, m0, -m1);
+    return order(g1, fmaf(2.f, g1, -m0));
+  };
+  auto same = [lo](float2 v) { return bc2(lo ? v.x : v.y); };
+  Mom e;
   if (kind == LBM_BC_EXTRAPOLATE) {
-    lbm::moments(m, c1, M1[0], M1[1], M1[2], M1[3], M1[4]);
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      G1[q] = 2.f * M0[q] - M1[q];
-      G2[q] = 2.f * G1[q] - M0[q];
-    }
-  } else {  // LBM_BC_REFLECT, normal velocity u1
-#pragma unroll
-    for (int q = 0; q < 5; ++q) G1[q] = G2[q] = M0[q];
-    G1[1] = 0.f;
-    G2[1] = -M0[1];
+    e.rho = ext(r.rho);
+    e.ux = ext(r.ux);
+    e.uy = ext(r.uy);
+    e.uz = ext(r.uz);
+    e.T = ext(r.T);
+  } else {  // LBM_BC_REFLECT
+    e.rho = same(r.rho);
+    e.ux = order(0.f, -(lo ? r.ux.x : r.ux.y));
+    e.uy = same(r.uy);
+    e.uz = same(r.uz);
+    e.T = same(r.T);
   }
-  lbm::equilibrium(m, G1[0], G1[1], G1[2], G1[3], G1[4], g1);
-  lbm::equilibrium(m, G2[0], G2[1], G2[2], G2[3], G2[4], g2);
+  e.usq = fma2(e.ux, e.ux, fma2(e.uy, e.uy, mul(e.uz, e.uz)));
+  return e;
+}
+
+// A layer of a reflecting y (AXIS 1) or z (AXIS 2) face from the moments r of
+// the pair at the face (Sec. 4(2)): the normal velocity 0 next to the face,
+// negated in the outer layer.
+template <int AXIS>
+__device__ __forceinline__ Mom wall_layer(const Mom& r, bool outer) {
+  Mom e = r;
+  float2& un = AXIS == 1 ? e.uy : e.uz;
+  un = outer ? neg(un) : make_float2(0.f, 0.f);
+  e.usq = fma2(e.ux, e.ux, fma2(e.uy, e.uy, mul(e.uz, e.uz)));
+  return e;
 }
 
 }  // namespace pm
