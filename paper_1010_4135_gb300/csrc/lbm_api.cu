@@ -341,6 +341,14 @@ unsigned fixed_faces(const lbm_sim* s) {
   return m;
 }
 
+// Bit a set where axis a is periodic.
+unsigned periodic_axes(const lbm_sim* s) {
+  unsigned p = 0;
+  for (int a = 0; a < 3; ++a)
+    if (s->bc.kind[2 * a] == LBM_BC_PERIODIC) p |= 1u << a;
+  return p;
+}
+
 // What the pair kernel does about the boundary layers (WtDesc).  `written`:
 // the faces whose layers it writes for the state it produces (periodic x for
 // even nx, where the boundary cell pairs are whole, and y, both from 4 cells
@@ -353,7 +361,12 @@ unsigned fixed_faces(const lbm_sim* s) {
 lbm::WtDesc write_through(const lbm_sim* s, unsigned* written, unsigned* own) {
   lbm::WtDesc w = {};
   *written = *own = 0;
-  if (s->prec != LBM_FP32 || !pair_variant(s->variant)) return w;
+  if (s->prec == LBM_FP64) {  // the FP64 kernel wraps periodic axes as it reads
+    for (int a = 0; a < 3; ++a)
+      if ((periodic_axes(s) >> a) & 1u) *own |= 3u << (2 * a);
+    return w;
+  }
+  if (!pair_variant(s->variant)) return w;
   const int* kind = s->bc.kind;
   const int nx = s->L.nx, ny = s->L.ny;
   if (wt_variant(s->variant)) {
@@ -608,9 +621,13 @@ int run_steps(lbm_sim* s, int64_t n) {
                    lbm::launch_step_tiled(s->scheme, s->tmap[s->cur], (const float*)fin, (float*)fout, s->L, s->mf,
                                           zc, s->flags, s->st));
       }
+    } else if (s->prec == LBM_FP32) {
+      LBM_LAUNCH(s, LBM_KERNEL_STEP,
+                 lbm::launch_step_plain(s->scheme, (const float*)fin, (float*)fout, s->L, s->mf, s->flags, s->st));
     } else {
       LBM_LAUNCH(s, LBM_KERNEL_STEP,
-                 lbm::launch_step_plain(s->prec, s->scheme, fin, fout, s->L, s->md, s->mf, s->flags, s->st));
+                 lbm::launch_step_fp64(s->scheme, (const double*)fin, (double*)fout, s->L, s->md, periodic_axes(s),
+                                       s->num_sms, s->flags, s->st));
     }
     s->layers_ok[s->cur ^ 1] = written ? 1 : 0;
     s->cur ^= 1;

@@ -10,6 +10,7 @@
 #include <cstdint>
 #include <cuda.h>
 #include <cuda_runtime.h>
+#include <utility>
 
 #include "lbm.h"
 
@@ -96,6 +97,32 @@ struct WtDesc {
   int per[3];
   int xlo, xhi, ylo, yhi, zlo, zhi;
 };
+
+// ---------------------------------------------------------------- launches
+
+// Programmatic dependent launch: a launch made by launch_chained
+// may start its CTAs once every CTA of the kernel before it in the stream has
+// called chain_start() (or ended), so the launch latency (2 to 4 us between
+// small dependent kernels) overlaps that kernel's end.  Such a kernel touches
+// no memory that other kernels use before chain_wait(), which waits until every
+// kernel before it has completed and its writes are visible.
+__device__ __forceinline__ void chain_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
 
 // ---------------------------------------------------------------- physics
 
@@ -185,26 +212,6 @@ __device__ __forceinline__ R clamp_mm(R x, R lo, R hi) {
   return fmin(fmax(x, lo), hi);
 }
 
-// minmod(x, d) of two doubles from their bit patterns, on the integer pipes:
-// 0 when the signs differ, else the operand of smaller magnitude (magnitudes
-// of IEEE doubles order like their bit patterns without the sign, compared
-// here as (high word, low word)).  The same value as the clamp form for
-// finite operands (a zero result may differ in sign).  GB300 executes FP64 at
-// a small fraction of its FP32 rate and a double min or max is an FP64
-// comparison, so the FP64 step kernel, bound by its FP64 pipe, takes its
-// minmods here.  Written on 32-bit halves: the same selection on 64-bit
-// integers cost the FP64 pipe 3 more instructions per gradient.
-__device__ __forceinline__ double minmod_bits(double x, double d) {
-  const int hx = __double2hiint(x), hd = __double2hiint(d);
-  const unsigned lx = (unsigned)__double2loint(x), ld = (unsigned)__double2loint(d);
-  const int mx = hx & 0x7fffffff, md = hd & 0x7fffffff;
-  const bool take_x = mx < md || (mx == md && lx <= ld);
-  const bool opposite = (hx ^ hd) < 0;
-  const int rh = opposite ? 0 : (take_x ? hx : hd);
-  const unsigned rl = opposite ? 0u : (take_x ? lx : ld);
-  return __hiloint2double(rh, (int)rl);
-}
-
 // dx * d(v f)/dx / v along one axis, from the upwind-side stencil:
 // v > 0 uses f at I-2..I+1 (m2, m1, c, p1); v < 0 uses I-1..I+2 (m1, c, p1, p2).
 // NND: (h_{I+1/2} - h_{I-1/2}) / v with the limited fluxes of Sec. 3; both
@@ -214,7 +221,6 @@ __device__ __forceinline__ R grad_pos(R m2, R m1, R c, R p1) {
   if (SCHEME == LBM_SCHEME_UPWIND1) return c - m1;
   if (SCHEME == LBM_SCHEME_UPWIND2) return R(0.5) * ((R(3) * c - R(4) * m1) + m2);
   const R d0 = c - m1;
-  if constexpr (sizeof(R) == 8) return d0 + R(0.5) * (minmod_bits(p1 - c, d0) - minmod_bits(m1 - m2, d0));
   const R lo = fmin(d0, R(0)), hi = fmax(d0, R(0));
   return d0 + R(0.5) * (clamp_mm(p1 - c, lo, hi) - clamp_mm(m1 - m2, lo, hi));
 }
@@ -223,7 +229,6 @@ __device__ __forceinline__ R grad_neg(R m1, R c, R p1, R p2) {
   if (SCHEME == LBM_SCHEME_UPWIND1) return p1 - c;
   if (SCHEME == LBM_SCHEME_UPWIND2) return R(0.5) * ((R(4) * p1 - R(3) * c) - p2);
   const R d1 = p1 - c;
-  if constexpr (sizeof(R) == 8) return d1 - R(0.5) * (minmod_bits(p2 - p1, d1) - minmod_bits(c - m1, d1));
   const R lo = fmin(d1, R(0)), hi = fmax(d1, R(0));
   return d1 - R(0.5) * (clamp_mm(p2 - p1, lo, hi) - clamp_mm(c - m1, lo, hi));
 }
@@ -245,8 +250,11 @@ cudaError_t launch_unpack(int prec, void* f, const Layout& L, const void* dense,
 cudaError_t launch_halo(int prec, void* f, const Layout& L, int side, int to_dense, void* dense, cudaStream_t st);
 cudaError_t launch_conserved(int prec, const void* f, const Layout& L, const Model<double>& m, double* partials,
                              int max_blocks, unsigned* counter, double* result, unsigned* flags, cudaStream_t st);
-cudaError_t launch_step_plain(int prec, int scheme, const void* fin, void* fout, const Layout& L,
-                              const Model<double>& md, const Model<float>& mf, unsigned* flags, cudaStream_t st);
+cudaError_t launch_step_plain(int scheme, const float* fin, float* fout, const Layout& L, const Model<float>& m,
+                              unsigned* flags, cudaStream_t st);
+// Double-precision step; `per`: bit a set where axis a is periodic (its layers are not read).
+cudaError_t launch_step_fp64(int scheme, const double* fin, double* fout, const Layout& L, const Model<double>& m,
+                             unsigned per, int num_sms, unsigned* flags, cudaStream_t st);
 cudaError_t launch_step_tiled(int scheme, const CUtensorMap& map, const float* fin, float* fout, const Layout& L,
                               const Model<float>& m, int zc, unsigned* flags, cudaStream_t st);
 // Pair kernel (two cells per thread) on `cols` x 8 tiles: cols = 64 (box
