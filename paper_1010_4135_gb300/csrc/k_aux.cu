@@ -83,6 +83,8 @@ __device__ __forceinline__ void fill_feq(const Model<float>& m, const float M[5]
 // type (the storage type of f: ghost values are stored at that precision).
 template <typename R, typename M>
 __global__ void fill_kernel(R* __restrict__ f, Layout L, Model<M> m, BcDesc bc, unsigned mask) {
+  chain_start();
+  chain_wait();
   const int face = blockIdx.y;
   if (!((mask >> face) & 1u)) return;
   const int axis = face >> 1, hi = face & 1;
@@ -396,9 +398,8 @@ cudaError_t launch_fill(int prec, void* f, const Layout& L, const Model<double>&
   for (int a = 0; a < 3; ++a)
     if (((mask >> (2 * a)) & 3u) && cnt[a] > cmax) cmax = cnt[a];
   dim3 grid((unsigned)((cmax + 127) / 128), 6);
-  if (prec == LBM_FP64) fill_kernel<double, double><<<grid, 128, 0, st>>>((double*)f, L, md, bc, mask);
-  else fill_kernel<float, float><<<grid, 128, 0, st>>>((float*)f, L, mf, bc, mask);
-  return cudaGetLastError();
+  if (prec == LBM_FP64) return launch_chained(fill_kernel<double, double>, grid, 128, 0, st, (double*)f, L, md, bc, mask);
+  return launch_chained(fill_kernel<float, float>, grid, 128, 0, st, (float*)f, L, mf, bc, mask);
 }
 
 cudaError_t launch_init(int prec, void* f, const Layout& L, const Model<double>& m, const double* rho, const double* u,

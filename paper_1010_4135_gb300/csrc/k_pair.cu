@@ -452,10 +452,12 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS_PER_SM)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
+  chain_wait();
   unsigned jb = 0;
   bool timed_out = false;
   pair_unit<SCHEME, G, O>(&tin, fin, fout, L, m, wt, rd, blockIdx.x * G::TX, blockIdx.y * G::TY, zs.z0(blockIdx.z),
                           zs.len(blockIdx.z, L.nz), flags, smem, bars, jb, timed_out, wait_limit);
+  chain_start();  // late: started early, the next step's CTAs pair up on the SMs that have room first
 }
 
 // Persistent batched step: two CTAs per SM take the units of every grid in
@@ -479,6 +481,7 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS_PER_SM)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
+  chain_wait();
   unsigned jb = 0;
   bool timed_out = false;
   __shared__ long long next;
@@ -507,6 +510,7 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS_PER_SM)
                             (t / it.tiles_x) * G::TY, zs.z0(chunk), zs.len(chunk, L.nz), it.flags, smem, bars, jb,
                             timed_out, tab.wait_limit);
   }
+  chain_start();
   if (threadIdx.x == 0) {
     __threadfence();
     if (atomicAdd(tab.done, 1u) == gridDim.x - 1) {
@@ -567,8 +571,8 @@ cudaError_t launch_scheme(const CUtensorMap& map, const float* fin, float* fout,
   Need need;
   need.add(L, G::TX, G::TY, m, wt, rd);
   with_form<SCHEME>(need, [&](auto o) {
-    step_pair_kernel<SCHEME, G, decltype(o)><<<grid, G::THREADS, G::SMEM, st>>>(map, fin, fout, L, m, wt, rd, zs, flags,
-                                                                                wait_limit);
+    launch_chained(step_pair_kernel<SCHEME, G, decltype(o)>, grid, G::THREADS, G::SMEM, st, map, fin, fout, L, m, wt, rd,
+                   zs, flags, wait_limit);
   });
   return cudaGetLastError();
 }
@@ -613,7 +617,7 @@ void launch_batch_scheme(const BatchTable& tab, int grid, cudaStream_t st) {
   for (int e = 0; e < tab.n; ++e)
     need.add(tab.item[e].L, G::TX, G::TY, tab.item[e].m, tab.item[e].wt, tab.item[e].rd);
   with_form<SCHEME>(need, [&](auto o) {
-    step_pair_batch_kernel<SCHEME, G, decltype(o)><<<grid, G::THREADS, G::SMEM, st>>>(tab);
+    launch_chained(step_pair_batch_kernel<SCHEME, G, decltype(o)>, grid, G::THREADS, G::SMEM, st, tab);
   });
 }
 
