@@ -96,10 +96,11 @@ using pm::ld2;
 // FULL: every tile lies inside the grid (nx and ny multiples of the tile), so
 // the activity tests fold away.  R1: dt = tau (dt/tau = 1, keep_2 = 0).  RD:
 // FP64 temperature recovery.  XF, WALL: layers of extrapolating / reflecting
-// x faces, of reflecting y and z faces, formed as they are read.
-template <bool FULL_, bool R1_, bool RD_, bool XF_, bool WALL_>
+// x faces, of reflecting y and z faces, formed as they are read.  FEW: fewer
+// than four rows and periodic y, so a row has several images.
+template <bool FULL_, bool R1_, bool RD_, bool XF_, bool WALL_, bool FEW_>
 struct Opt {
-  static constexpr bool FULL = FULL_, R1 = R1_, RD = RD_, XF = XF_, WALL = WALL_;
+  static constexpr bool FULL = FULL_, R1 = R1_, RD = RD_, XF = XF_, WALL = WALL_, FEW = FEW_;
 };
 
 // Named barrier `id` over 128 threads with an OR of v across them.
@@ -241,10 +242,11 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* _
   // T makes the sum non-finite, and so does a non-finite velocity: T is
   // (E/rho - u^2)/b, -inf or NaN when u^2 is inf or NaN.
   float2 hmin_rho = make_float2(INFINITY, INFINITY), hmin_T = hmin_rho, hsum = make_float2(0.f, 0.f);
-  // periodic images of this pair (element offsets from its own index, 0 = none)
+  // periodic images of this pair (element offsets from its own index, 0 = none):
+  // one per axis, or with fewer than four rows (FEW) several y ones
   unsigned img_y = 0, img_x = 0;
   if (act0) {
-    if (wt.per[1]) img_y = (unsigned)L.sx * (unsigned)(y < 2 ? L.ny : (y >= L.ny - 2 ? -L.ny : 0));
+    if (!O::FEW && wt.per[1]) img_y = (unsigned)L.sx * (unsigned)(y < 2 ? L.ny : (y >= L.ny - 2 ? -L.ny : 0));
     if (wt.per[0]) img_x = (unsigned)(x == 0 ? L.nx : (x == L.nx - 2 ? -L.nx : 0));
   }
   // store the pair's new values of plane k, the deferred fields (late) or the others, and their images
@@ -267,6 +269,12 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* _
     if (img_y | img_x) {
       if (img_y) put(g + img_y);
       if (img_x) put(g + img_x);
+    }
+    if (O::FEW && wt.per[1] && act0) {
+#pragma unroll 1
+      for (int q = -2; q < L.ny + 2; ++q)
+        if (q < 0 || q >= L.ny)
+          if ((q - y) % L.ny == 0) put(g + (unsigned)(q - y) * (unsigned)L.sx);
     }
   };
   // faces whose layers are formed here, from the moments of the cells at the
@@ -523,29 +531,32 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS_PER_SM)
 
 // What the forms go by, over all grids of a launch.
 struct Need {
-  bool full = true, r1 = true, rd = false, xf = false, wall = false;
+  bool full = true, r1 = true, rd = false, xf = false, wall = false, few = false;
   void add(const Layout& L, int tx, int ty, const Model<float>& m, const WtDesc& wt, const RecoverDesc& r) {
     full = full && L.nx % tx == 0 && L.ny % ty == 0;
     r1 = r1 && m.dt_tau == 1.0f && m.keep2 == 0.0f;
     rd = rd || r.on;
     xf = xf || wt.xlo || wt.xhi;
     wall = wall || wt.ylo || wt.yhi || wt.zlo || wt.zhi;
+    few = few || (wt.per[1] && L.ny < 4);
   }
 };
 
 // The forms that exist: NND with dt = tau and no recovery (every run of the
 // paper) has one per boundary need, everything else one form with all parts.
-using FullPlain = Opt<true, true, false, false, false>;
-using FullFaces = Opt<true, true, false, true, false>;
-using Plain = Opt<false, true, false, false, false>;
-using Faces = Opt<false, true, false, true, false>;
-using Walls = Opt<false, true, false, true, true>;
-using General = Opt<false, false, true, true, true>;
+using FullPlain = Opt<true, true, false, false, false, false>;
+using FullFaces = Opt<true, true, false, true, false, false>;
+using Plain = Opt<false, true, false, false, false, false>;
+using Faces = Opt<false, true, false, true, false, false>;
+using Walls = Opt<false, true, false, true, true, false>;
+using FewRows = Opt<false, true, false, true, false, true>;
+using General = Opt<false, false, true, true, true, true>;
 
 template <int SCHEME, class F>
 void with_form(const Need& n, F f) {
   if constexpr (SCHEME == LBM_SCHEME_NND) {
-    if (n.r1 && !n.rd) {
+    if (n.r1 && !n.rd && !(n.few && n.wall)) {
+      if (n.few) return f(FewRows());
       if (n.wall) return f(Walls());
       if (n.full) return n.xf ? f(FullFaces()) : f(FullPlain());
       return n.xf ? f(Faces()) : f(Plain());
@@ -592,7 +603,7 @@ cudaError_t launch_geo(int scheme, const CUtensorMap& map, const float* fin, flo
 
 template <class G>
 cudaError_t prepare_geo() {
-  cudaError_t e = set_attributes<LBM_SCHEME_NND, G, FullPlain, FullFaces, Plain, Faces, Walls, General>();
+  cudaError_t e = set_attributes<LBM_SCHEME_NND, G, FullPlain, FullFaces, Plain, Faces, Walls, FewRows, General>();
   if (e == cudaSuccess) e = set_attributes<LBM_SCHEME_UPWIND2, G, General>();
   if (e == cudaSuccess) e = set_attributes<LBM_SCHEME_UPWIND1, G, General>();
   return e;

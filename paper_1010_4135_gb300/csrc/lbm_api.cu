@@ -308,24 +308,61 @@ bool pair_variant(int variant) {
 }
 int pair_cols(int variant) { return variant == LBM_VARIANT_TILED64 ? 64 : 32; }
 
-// z planes per CTA of the tiled kernels (`cols` x 8 tiles, `ctas` CTAs per
-// SM) when none is set: the largest of 32, 24, 16, 12, 8, 6, 4 that still
-// gives two waves of units.  Each unit re-reads four planes around its chunk
-// and pays a prologue, so long chunks save work; short chunks fill the SMs.
-// The pair kernels then end each column in 8-plane chunks (auto_ztail), so
-// the last wave is short.  Measured on GB300 (32 x 8 tiles): 256^3 gets 32 + 8
-// (0.464-0.469 ms; equal 16 / 24 / 32: 0.481 / 0.472 / 0.482), 192^3 32 + 8
-// (0.218; best measured 0.216), 128^3 12 + 8 (equal 12: 0.085).  The
-// autotuner (autotune.py) measures the choice per grid.
-int auto_zchunk(const Layout& L, int num_sms, int cols, int ctas) {
-  const long long tiles = (long long)((L.nx + cols - 1) / cols) * ((L.ny + lbm::kTileY - 1) / lbm::kTileY);
-  const long long want = 2LL * ctas * num_sms;
+// z planes per CTA of the single-cell tiled kernel when none is set: the
+// largest of 32, 24, 16, 12, 8, 6, 4 that still gives two waves of units.
+int auto_zchunk(const Layout& L, int num_sms) {
+  const long long tiles = (long long)((L.nx + lbm::kTileX - 1) / lbm::kTileX) * ((L.ny + lbm::kTileY - 1) / lbm::kTileY);
+  const long long want = 4LL * num_sms;
   static const int cand[] = {32, 24, 16, 12, 8, 6, 4};
   for (int zc : cand)
     if (tiles * ((L.nz + zc - 1) / zc) >= want) return zc < L.nz ? zc : L.nz;
   return L.nz < 4 ? L.nz : 4;
 }
-int auto_ztail(int zc) { return zc >= 12 ? 8 : 0; }
+
+// Chunks of the pair kernel when none are set, from the planes per CTA slot
+// (two slots per SM), r = tiles nz / slots.
+// r < 12: equal chunks.  A unit takes its planes and about 1.5 planes' time
+// to start; a plane takes about 1.45 us on an SM with one unit and 1.95 us
+// where two share it.  The chunk with the least time for all waves by these
+// figures (200 x 4 x 4 one plane, 3.7 us against 7.3 with four; 96^3 12
+// planes, exactly 288 units, 29.6 against 37.2 with four).
+// r <= 80: as many long chunks per column as w waves of slots hold, w =
+// ceil(r / 45), each 0.95 r / w planes as far as that number allows, and the
+// rest of the column in 4-plane chunks that fill the slots left (128^3: 26 + 4,
+// 59.9 us, 12 + 8 68.9, one more long chunk per column, 24 + 4, 79.7;
+// 192 x 128 x 128: 36 + 4, 82.8 against 89.5).
+// Beyond, 32 planes ending in 8-plane chunks: the re-read planes at the chunks'
+// ends count more than the last wave (256^3 383 us, the best of 60 379).
+lbm::ZSched auto_zsched(const Layout& L, int num_sms, const lbm::PairShape& shape) {
+  const int slots = shape.ctas_per_sm * num_sms;
+  const long long tiles = (long long)((L.nx + shape.tx - 1) / shape.tx) * ((L.ny + shape.ty - 1) / shape.ty);
+  const double r = (double)tiles * L.nz / slots;
+  if (r > 80.0) return lbm::make_zsched(L.nz, 32, 8);
+  if (r >= 12.0) {
+    const int w = (int)std::ceil(r / 45.0);
+    const int nl = (int)((long long)w * slots / tiles);
+    if (nl >= 1 && L.nz > 4) {
+      const int lo = (L.nz - 4) / (nl + 1) + 1, hi = (L.nz - 4) / nl;
+      int zc = (int)std::lround(0.95 * r / w);
+      if (zc > hi) zc = hi;
+      if (zc < lo) zc = lo;
+      return lbm::make_zsched(L.nz, zc, 4);
+    }
+    return lbm::make_zsched(L.nz, 32, 8);
+  }
+  int best = 1;
+  double least = 0.0;
+  for (int zc = 1; zc <= L.nz && zc <= 24; ++zc) {
+    const double planes = zc + 1.5;
+    const long long units = tiles * ((L.nz + zc - 1) / zc), rem = units % slots;
+    const double t = (units / slots) * planes * 1.95 + (rem == 0 ? 0.0 : planes * (rem <= num_sms ? 1.45 : 1.95));
+    if (zc == 1 || t < least) {
+      least = t;
+      best = zc;
+    }
+  }
+  return lbm::make_zsched(L.nz, best, 0);
+}
 
 unsigned step_faces(const lbm_sim* s) {
   unsigned m = 0;
@@ -350,9 +387,9 @@ unsigned periodic_axes(const lbm_sim* s) {
 }
 
 // What the pair kernel does about the boundary layers (WtDesc).  `written`:
-// the faces whose layers it writes for the state it produces (periodic x for
-// even nx, where the boundary cell pairs are whole, and y, both from 4 cells
-// on, where a cell has one image per axis); `own`: the faces whose layers it
+// the faces whose layers it writes for the state it produces (periodic y, and
+// x for even nx, where the boundary cell pairs are whole, from 4 cells on,
+// where a pair has one image); `own`: the faces whose layers it
 // never reads (periodic z; extrapolating and reflecting x faces, of which the
 // hi one needs a whole cell pair, nx even; reflecting y and z faces, of which
 // the y-hi one needs its row and the one before in one warp, ny even; none
@@ -371,7 +408,7 @@ lbm::WtDesc write_through(const lbm_sim* s, unsigned* written, unsigned* own) {
   const int nx = s->L.nx, ny = s->L.ny;
   if (wt_variant(s->variant)) {
     w.per[0] = kind[0] == LBM_BC_PERIODIC && nx >= 4 && nx % 2 == 0;
-    w.per[1] = kind[2] == LBM_BC_PERIODIC && ny >= 4;
+    w.per[1] = kind[2] == LBM_BC_PERIODIC;
     w.per[2] = kind[4] == LBM_BC_PERIODIC;
     if (w.per[0]) *written |= 3u;
     if (w.per[1]) *written |= 3u << 2;
@@ -607,16 +644,15 @@ int run_steps(lbm_sim* s, int64_t n) {
     if (mask)
       LBM_LAUNCH(s, LBM_KERNEL_FILL, lbm::launch_fill(s->prec, fin, s->L, s->md, s->mf, s->bc, mask, s->st));
     if (s->prec == LBM_FP32 && s->variant != LBM_VARIANT_PLAIN) {
-      const int zc = s->zchunk > 0 ? s->zchunk
-                                   : (pair ? auto_zchunk(s->L, s->num_sms, shape.tx, shape.ctas_per_sm)
-                                           : auto_zchunk(s->L, s->num_sms, lbm::kTileX, 2));
       if (pair) {
         const CUtensorMap& map = shape.tx == 64 ? s->wmap[s->cur] : s->tmap[s->cur];
-        const lbm::ZSched zs = lbm::make_zsched(s->L.nz, zc, s->zchunk > 0 ? s->ztail : auto_ztail(zc));
+        const lbm::ZSched zs = s->zchunk > 0 ? lbm::make_zsched(s->L.nz, s->zchunk, s->ztail)
+                                             : auto_zsched(s->L, s->num_sms, shape);
         LBM_LAUNCH(s, LBM_KERNEL_STEP,
                    lbm::launch_step_pair(shape.tx, s->scheme, map, (const float*)fin, (float*)fout, s->L, s->mf, wt,
                                          s->rd, zs, s->flags, s->wait_limit, s->st));
       } else {
+        const int zc = s->zchunk > 0 ? s->zchunk : auto_zchunk(s->L, s->num_sms);
         LBM_LAUNCH(s, LBM_KERNEL_STEP,
                    lbm::launch_step_tiled(s->scheme, s->tmap[s->cur], (const float*)fin, (float*)fout, s->L, s->mf,
                                           zc, s->flags, s->st));
@@ -636,10 +672,18 @@ int run_steps(lbm_sim* s, int64_t n) {
   return LBM_OK;
 }
 
-// z planes per unit of the batched kernel when a sim has none set.  Measured
-// (GB300): eight 128^3 grids 0.526 / 0.522 / 0.529 ms per step at 16 / 24 / 32
-// planes; with the 512 x 256 x 256 grid added 1.430 / 1.394 / 1.386 ms.
-constexpr int kBatchZchunk = 24;
+// Chunks of the batched kernel for sims with none set, from the planes per CTA
+// slot over all grids, r: units come from one queue, so only the last ones
+// leave slots idle, and about 1.7 sqrt(r) planes balance that against the time
+// a unit takes to start (us per step: two 64^3 grids, r = 7, 4 planes 29.1, 8
+// 30.5, 24 64.7; eight 64^3, r = 27, 8 + 0 89.4, 24 109; four grids of 64^3 to
+// 192 x 128 x 128, r = 82, 14 + 8 193, 24 202; eight 128^3, r = 216, 28 463, 16
+// 471; with 512 x 256 x 256, r = 647, 32 1231, 24 1247, 16 1283).
+lbm::ZSched batch_zsched(int nz, double r) {
+  int zc = (int)std::lround(1.7 * std::sqrt(r));
+  zc = zc < 2 ? 2 : (zc > 32 ? 32 : zc);
+  return lbm::make_zsched(nz, zc, zc >= 10 && zc <= 20 ? 8 : 0);
+}
 
 int batch_check(lbm_sim* const* sims, int32_t n) {
   if (!sims || n < 1 || n > lbm::kMaxBatch) return LBM_EINVAL;
@@ -668,7 +712,12 @@ int run_batch(lbm_sim* const* sims, int32_t n, int64_t steps) {
   thread_local static lbm::BatchTable tab;  // built on the host, passed by value to the kernel
   unsigned written[lbm::kMaxBatch], own[lbm::kMaxBatch];
   lbm::WtDesc wt[lbm::kMaxBatch];
-  for (int i = 0; i < n; ++i) wt[i] = write_through(sims[i], &written[i], &own[i]);
+  double planes = 0.0;  // tile planes of all grids
+  for (int i = 0; i < n; ++i) {
+    const Layout& L = sims[i]->L;
+    wt[i] = write_through(sims[i], &written[i], &own[i]);
+    planes += (double)((L.nx + shape.tx - 1) / shape.tx) * ((L.ny + shape.ty - 1) / shape.ty) * L.nz;
+  }
   for (int64_t k = 0; k < steps; ++k) {
     long long units = 0;
     for (int i = 0; i < n; ++i) {
@@ -690,7 +739,7 @@ int run_batch(lbm_sim* const* sims, int32_t n, int64_t steps) {
       it.tiles_x = (s->L.nx + shape.tx - 1) / shape.tx;
       it.tiles_y = (s->L.ny + shape.ty - 1) / shape.ty;
       it.zs = s->zchunk > 0 ? lbm::make_zsched(s->L.nz, s->zchunk, s->ztail)
-                            : lbm::make_zsched(s->L.nz, kBatchZchunk, 0);
+                            : batch_zsched(s->L.nz, planes / ((double)shape.ctas_per_sm * s0->num_sms));
       it.first_unit = units;
       units += (long long)it.tiles_x * it.tiles_y * it.zs.nch;
     }

@@ -34,6 +34,9 @@ GRIDS = {
     "periodic_z1": ((32, 16, 1), (F, P, P), (E, P, P)),
     "periodic_z2": ((33, 5, 2), (P, P, P), (P, P, P)),
     "periodic_z3": ((40, 3, 3), (P, P, P), (P, P, P)),
+    "one_row": ((33, 1, 4), (F, P, P), (E, P, P)),
+    "two_rows": ((64, 2, 5), (F, P, P), (F, P, P)),
+    "three_rows_and_walls": ((34, 3, 6), (E, P, R), (F, P, R)),
     "mixed_walls": ((64, 8, 13), (F, R, E), (E, F, R)),
 }
 
