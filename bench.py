@@ -228,7 +228,7 @@ def measured_peak():
 # these files are unchanged
 KERNEL_SOURCES = {
     "step_fp32": ("k_pair.cu", "pair_math.cuh", "tma_ring.cuh", "lbm_internal.cuh"),
-    "step_fp64": ("k_plain.cu", "lbm_internal.cuh"),
+    "step_fp64": ("k_plain.cu", "fixed_sum.cuh", "lbm_internal.cuh"),
 }
 
 

@@ -2,56 +2,55 @@
 // conservation reduction.  Initialisation and moments compute in double
 // precision whatever the storage type of f; the boundary fill computes in the
 // storage precision (its results are stored at that precision).
+#include "fixed_sum.cuh"
 #include "pair_math.cuh"
 
 namespace lbm {
 namespace {
 
-template <typename R>
-__device__ __forceinline__ void load_cell(const R* __restrict__ f, long long fs, long long idx, double v[NV]) {
-#pragma unroll
-  for (int i = 0; i < NV; ++i) v[i] = (double)f[i * fs + idx];
+// A double rounded to the nearest float (ties to even) on the integer ALUs:
+// the conversion instruction runs on the FP64 pipe, which bounds the kernels
+// here.  Values outside the normal float range take the instruction.
+__device__ __noinline__ float narrow_any(double v) { return (float)v; }  // out of line: inline it would run always
+__device__ __forceinline__ double narrow(double v, double) { return v; }
+__device__ __forceinline__ float narrow(double v, float) {
+  const int h = __double2hiint(v);
+  const unsigned l = (unsigned)__double2loint(v);
+  const unsigned m = (unsigned)h & 0x7fffffffu;
+  if (m < (897u << 20) || m >= (1150u << 20)) return narrow_any(v);  // below 2^-126, or 2^127 and above
+  const unsigned b = __funnelshift_l(l, m - (896u << 20), 3);
+  const unsigned r = b + (((l & 0x1fffffffu) + 0x0fffffffu + (b & 1u)) >> 29);
+  return __uint_as_float(r | ((unsigned)h & 0x80000000u));
 }
 
 template <typename R>
 __device__ __forceinline__ void store_cell(R* __restrict__ f, long long fs, long long idx, const double v[NV]) {
 #pragma unroll
-  for (int i = 0; i < NV; ++i) f[i * fs + idx] = (R)v[i];
+  for (int i = 0; i < NV; ++i) f[i * fs + idx] = narrow(v[i], R());
 }
 
-__device__ __forceinline__ void macros_at(const Model<double>& m, const double v[NV], double out[5]) {
-  double rho, ux, uy, uz, T;
-  moments(m, v, rho, ux, uy, uz, T);
-  out[0] = rho; out[1] = ux; out[2] = uy; out[3] = uz; out[4] = T;
-}
-
-// Error-free sum of two floats: s + e == a + b exactly.
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = a + b;
-  const float bp = s - a;
-  e = (a - (s - bp)) + (b - bp);
-}
-
-// Running sum of floats held as an unevaluated pair hi + lo (about 44
-// significant bits).  add() keeps hi the rounded running sum and adds its
-// rounding error (exact, two_sum) to lo; renorm() folds lo back into hi
-// (|hi| >= |lo|, so the fast two-sum is exact) and is called every few adds,
-// so lo stays of order 2^-24 |hi| and n additions lose about n * 2^-48
-// relative.
-struct DFloat {
-  float hi = 0.f, lo = 0.f;
-  __device__ __forceinline__ void add(float x) {
-    float s, e;
-    two_sum(hi, x, s, e);
+// Running sums of two float lanes, each held as an unevaluated pair hi + lo
+// (about 44 significant bits), in packed arithmetic.  add() keeps hi the
+// rounded running sum and adds its rounding error (exact: the error-free sum
+// of two floats) to lo; renorm() folds lo back into hi (|hi| >= |lo|, so the
+// fast two-sum is exact) and is called every few adds, so lo stays of order
+// 2^-24 |hi| and n additions lose about n * 2^-48 relative.
+struct DFloat2 {
+  float2 hi = {0.f, 0.f}, lo = {0.f, 0.f};
+  __device__ __forceinline__ void add(float2 x) {
+    const float2 s = pm::add(hi, x), bp = pm::sub(s, hi);
+    const float2 e = pm::add(pm::sub(hi, pm::sub(s, bp)), pm::sub(x, bp));
     hi = s;
-    lo += e;
+    lo = pm::add(lo, e);
   }
   __device__ __forceinline__ void renorm() {
-    const float s = hi + lo;
-    lo = lo - (s - hi);
+    const float2 s = pm::add(hi, lo);
+    lo = pm::sub(lo, pm::sub(s, hi));
     hi = s;
   }
-  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+  __device__ __forceinline__ double value() const {
+    return ((double)hi.x + (double)lo.x) + ((double)hi.y + (double)lo.y);
+  }
 };
 
 // Moments and equilibrium of the boundary fill.  In single precision they are
@@ -151,11 +150,41 @@ __global__ void fill_kernel(R* __restrict__ f, Layout L, Model<M> m, BcDesc bc, 
 
 __device__ __forceinline__ bool cell_of(const Layout& L, long long k, int& x, int& y, int& z) {
   if (k >= L.ncell()) return false;
-  x = (int)(k % L.nx);
-  const long long r = k / L.nx;
-  y = (int)(r % L.ny);
-  z = (int)(r / L.ny);
+  const unsigned q = (unsigned)k, r = q / (unsigned)L.nx;  // a field has fewer than 2^32 cells
+  x = (int)(q - r * (unsigned)L.nx);
+  z = (int)(r / (unsigned)L.ny);
+  y = (int)(r - (unsigned)z * (unsigned)L.ny);
   return true;
+}
+
+// f^eq of one cell in double precision (Eq. "eq"), rho folded into the
+// shells' coefficients and opposite velocities sharing their even part: 60
+// FP64 operations against 77 velocity by velocity.
+__device__ __forceinline__ void feq_fp64(const Model<double>& m, double rho, double ux, double uy, double uz, double T,
+                                         double e[NV]) {
+  const double usq = fma(ux, ux, fma(uy, uy, uz * uz));
+  e[0] = rho * (m.AR * T);
+  {
+    const double rA = rho * fma(m.AaT, T, fma(m.AaU, usq, m.Aa0)), rB = rho * fma(m.BaT, T, fma(m.BaU, usq, m.Ba0));
+    const double rD = rho * m.Da;
+    const double u3[3] = {ux, uy, uz};
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const double w = m.c1 * u3[a], q = fma(rD, w * w, rA);
+      e[1 + 2 * a] = fma(rB, w, q);
+      e[2 + 2 * a] = fma(-rB, w, q);
+    }
+  }
+  const double rA = rho * fma(m.AdT, T, fma(m.AdU, usq, m.Ad0)), rB = rho * fma(m.BdT, T, fma(m.BdU, usq, m.Bd0));
+  const double rD = rho * m.Dd;
+  const double sxy = ux + uy, dxy = ux - uy;
+  const double t4[4] = {sxy + uz, sxy - uz, dxy + uz, dxy - uz};
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const double w = m.s * t4[k], q = fma(rD, w * w, rA);
+    e[7 + k] = fma(rB, w, q);
+    e[14 - k] = fma(-rB, w, q);
+  }
 }
 
 template <typename R>
@@ -166,25 +195,31 @@ __global__ void init_kernel(R* __restrict__ f, Layout L, Model<double> m, const 
   if (!cell_of(L, k, x, y, z)) return;
   const long long n = L.ncell();
   double e[NV];
-  equilibrium(m, rho[k], u[k], u[n + k], u[2 * n + k], T[k], e);
+  feq_fp64(m, rho[k], u[k], u[n + k], u[2 * n + k], T[k], e);
   store_cell(f, L.fs, L.at(x, y, z), e);
 }
 
+// One thread per cell; the sums run in fixed point (fixed_sum.cuh), so of the
+// FP64 pipe's work the 15 conversions from float and half of the moments'
+// operations go.
 template <typename R>
-__global__ void moments_kernel(const R* __restrict__ f, Layout L, Model<double> m, double* __restrict__ rho,
-                               double* __restrict__ u, double* __restrict__ T) {
+__global__ void __launch_bounds__(256) moments_kernel(const R* __restrict__ f, Layout L, Model<double> m,
+                                                      double* __restrict__ rho, double* __restrict__ u,
+                                                      double* __restrict__ T) {
   const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   int x, y, z;
   if (!cell_of(L, k, x, y, z)) return;
-  const long long n = L.ncell();
-  double v[NV], mm[5];
-  load_cell(f, L.fs, L.at(x, y, z), v);
-  macros_at(m, v, mm);
-  rho[k] = mm[0];
-  u[k] = mm[1];
-  u[n + k] = mm[2];
-  u[2 * n + k] = mm[3];
-  T[k] = mm[4];
+  const long long n = L.ncell(), at = L.at(x, y, z);
+  R v[NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) v[i] = f[i * L.fs + at];
+  double r, ux, uy, uz, t;
+  fx::moments_fixed(m, v, r, ux, uy, uz, t);
+  rho[k] = r;
+  u[k] = ux;
+  u[n + k] = uy;
+  u[2 * n + k] = uz;
+  T[k] = t;
 }
 
 template <typename R>
@@ -231,35 +266,54 @@ constexpr int RED_GROUPS = 3, RED_GF = NV / RED_GROUPS, RED_ROWS = 4;
 constexpr int RED_THREADS = 32 * RED_GROUPS * RED_ROWS;
 static_assert(RED_GROUPS * RED_GF == NV, "field groups cover the 15 fields");
 
-__device__ __forceinline__ bool finite_value(double v) { return fabs(v) < 1e300; }
-__device__ __forceinline__ bool finite_value(float v) { return fabsf(v) < 3.0e38f; }
-
-// Per-field accumulation of one thread's cells: double for double storage;
-// for float storage an error-free double-float pair, converted to double at
-// the end (GB300's FP64 rate would make a per-value conversion and double
-// add the bottleneck of this memory-bound reduction).
+// Per-field accumulation of one thread's cells, four floats or two doubles at
+// a time: double for double storage; for float storage error-free double-float
+// pairs, converted to double at the end (GB300's FP64 rate would make a
+// per-value conversion and double add the bottleneck of this memory-bound
+// reduction).  `largest` follows the values' magnitudes, on the integer ALUs
+// for doubles (a double comparison runs on the FP64 pipe); a NaN shows in the
+// sum.
 template <typename R, int N>
 struct FieldAcc;
 template <int N>
 struct FieldAcc<double, N> {
   double s[N];
+  int largest = 0;
   __device__ FieldAcc() {
 #pragma unroll
     for (int i = 0; i < N; ++i) s[i] = 0.0;
   }
-  __device__ __forceinline__ void add(int i, double v) { s[i] += v; }
+  __device__ __forceinline__ void add(int i, const double v[2]) {
+    s[i] += v[0];
+    s[i] += v[1];
+    largest = max(largest, max(fx::mag(v[0]), fx::mag(v[1])));
+  }
   __device__ __forceinline__ void renorm() {}
   __device__ __forceinline__ double value(int i) const { return s[i]; }
+  // a NaN or infinity has a high word above every finite one
+  __device__ __forceinline__ bool bad() const { return !(__hiloint2double(largest, 0) < 1e300); }
 };
 template <int N>
 struct FieldAcc<float, N> {
-  DFloat s[N];
-  __device__ __forceinline__ void add(int i, float v) { s[i].add(v); }
+  DFloat2 s[N];
+  float largest = 0.f;
+  __device__ __forceinline__ void add(int i, const float v[4]) {
+    s[i].add(make_float2(v[0], v[1]));
+    s[i].add(make_float2(v[2], v[3]));
+#pragma unroll
+    for (int k = 0; k < 4; ++k) largest = fmaxf(largest, fabsf(v[k]));
+  }
   __device__ __forceinline__ void renorm() {
 #pragma unroll
     for (int i = 0; i < N; ++i) s[i].renorm();
   }
   __device__ __forceinline__ double value(int i) const { return s[i].value(); }
+  __device__ __forceinline__ bool bad() const {
+    bool nan = false;
+#pragma unroll
+    for (int i = 0; i < N; ++i) nan = nan || isnan(s[i].hi.x + s[i].lo.x) || isnan(s[i].hi.y + s[i].lo.y);
+    return nan || !(largest < 3.0e38f);
+  }
 };
 
 // 16-byte vector loads of float / double rows (read once: streaming hint).
@@ -297,7 +351,6 @@ __global__ void __launch_bounds__(RED_THREADS) conserved_kernel(const R* __restr
   __shared__ double part[16][16];
   __shared__ bool last;
   FieldAcc<R, RED_GF> acc;
-  bool bad = false;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int grp = warp % RED_GROUPS, slot = warp / RED_GROUPS;
   const int nrows = L.ny * L.nz;
@@ -313,19 +366,19 @@ __global__ void __launch_bounds__(RED_THREADS) conserved_kernel(const R* __restr
       R v[RED_GF][VW];
 #pragma unroll
       for (int i = 0; i < RED_GF; ++i) load16(row + i * L.fs + x0, v[i]);
+      if (x0 + VW > L.nx) {
 #pragma unroll
-      for (int i = 0; i < RED_GF; ++i) {
+        for (int i = 0; i < RED_GF; ++i)
 #pragma unroll
-        for (int k = 0; k < VW; ++k) {
-          const R e = x0 + k < L.nx ? v[i][k] : R(0);
-          bad |= !finite_value(e);
-          acc.add(i, e);
-        }
+          for (int k = 0; k < VW; ++k)
+            if (x0 + k >= L.nx) v[i][k] = R(0);
       }
+#pragma unroll
+      for (int i = 0; i < RED_GF; ++i) acc.add(i, v[i]);
       acc.renorm();
     }
   }
-  if (bad) atomicOr(flags, (unsigned)LBM_HEALTH_NONFINITE);
+  if (acc.bad()) atomicOr(flags, (unsigned)LBM_HEALTH_NONFINITE);
 #pragma unroll
   for (int i = 0; i < RED_GF; ++i) {
     double v = acc.value(i);
@@ -441,7 +494,9 @@ cudaError_t launch_halo(int prec, void* f, const Layout& L, int side, int to_den
 
 cudaError_t launch_conserved(int prec, const void* f, const Layout& L, const Model<double>& m, double* partials,
                              int max_blocks, unsigned* counter, double* result, unsigned* flags, cudaStream_t st) {
-  // about eight rows per row slot, at most max_blocks blocks
+  // about eight rows per row slot, and no more blocks than run at once: a
+  // block's reduction at its end is some 300 FP64 operations per warp (256^3
+  // FP32, us per call: 2048 blocks 287, 455 blocks 239)
   int b = blocks_for((long long)L.ny * L.nz, 8 * RED_ROWS);
   if (b > max_blocks) b = max_blocks;
   if (b < 1) b = 1;

@@ -4,7 +4,7 @@
 // Laplacian (i = 0..6) -> BGK + forward Euler, written to fout.
 // step_plain_kernel is the single-precision cross-check variant;
 // step_fp64_kernel is the double-precision path.
-#include "lbm_internal.cuh"
+#include "fixed_sum.cuh"
 
 namespace lbm {
 namespace {
@@ -75,51 +75,17 @@ __global__ void __launch_bounds__(256) step_plain_kernel(const float* __restrict
 // FP32 or integer ones, so the step is bound by the FP64 operations it needs
 // and everything linear in f is taken off that pipe: the moments' sums, the
 // convection's differences, minmods and sums, and the Laplacian, run in 64-bit
-// integers.  The values of one sum (a velocity's stencil, or a cell's 15
-// values) are aligned to the largest exponent among them, E: v = n 2^(E -
-// 1079), |n| < 2^57, which holds all 53 bits of values down to 2^-4 of the
-// largest and truncates smaller ones below 2^-56 of it.  The largest sum, five
-// times twice the convection of an axis velocity (|difference| <= 2, |minmod|
-// <= |difference|) less its Laplacian, is at most 52 times the largest value
-// (a diagonal velocity's convection 24 times), so 63 bits hold it and every
-// difference, minmod and sum is exact; each sum is rounded once, to 53 bits,
-// when it becomes a double.  A double evaluation rounds at each of these
-// operations, at 2^-53 of the operands.  Sums whose largest exponent is
-// outside [EMIN, EMAX] (non-finite, or beyond 1e-247 .. 1e264) take a double
-// evaluation.  256^3: 13.3 -> 4.4 ms per step (417 -> about 130 FP64 operations
-// per cell; the FP64 pipe 84 -> 67 % busy, the integer ALUs 74 %: both near
-// their rates); 300 x 80 x 80 with walls 1.68 -> 0.58 ms.
-constexpr int EMIN = 200, EMAX = 1900;
-constexpr int FX_SHIFT = 4;                      // 53-bit mantissas, top bit at bit 56
-constexpr int FX_BIAS = 1023 + 52 + FX_SHIFT;    // n counts units of 2^(E - FX_BIAS)
-
-__device__ __forceinline__ int mag_hi(double v) { return __double2hiint(v) & 0x7fffffff; }
-
-// v in units of 2^(E - FX_BIAS), truncated toward zero; E >= EMIN is at least
-// v's exponent (zeros and subnormals are shifted out).
-__device__ __forceinline__ long long to_fixed(double v, int E) {
-  const int h = __double2hiint(v);
-  const unsigned l = (unsigned)__double2loint(v);
-  unsigned long long n = (((unsigned long long)(((unsigned)h & 0xfffffu) | 0x100000u) << 32) | l) << FX_SHIFT;
-  const unsigned sh = (unsigned)(E - (mag_hi(v) >> 20));
-  asm("shr.u64 %0, %0, %1;" : "+l"(n) : "r"(sh));  // PTX clamps the shift at 64
-  const long long s = h >> 31;
-  return ((long long)n ^ s) - s;
-}
-
-// n 2^(E - FX_BIAS), rounded to 53 bits (a tie away from zero).
-__device__ __forceinline__ double from_fixed(long long n, int E) {
-  const long long s = n >> 63;
-  unsigned long long a = (unsigned long long)((n ^ s) - s);
-  const int lz = __clzll((long long)a);
-  a = a << (lz & 63);
-  // top bit 63 - lz: biased exponent E - FX_BIAS + 1023 + 63 - lz, less one for
-  // the mantissa's leading bit, which the sum below adds to it
-  const unsigned e = (unsigned)(E - FX_BIAS + 1023 + 62 - lz);
-  const unsigned long long q = (a >> 11) + ((a >> 10) & 1ull);  // a carry to 2^53 raises the exponent
-  const unsigned hi = ((unsigned)(q >> 32) + (e << 20)) | ((unsigned)(s >> 32) & 0x80000000u);
-  return a == 0 ? 0.0 : __hiloint2double((int)hi, (int)(unsigned)q);
-}
+// fixed point (fixed_sum.cuh; the values aligned are a velocity's stencil, or
+// a cell's 15 values).  The largest sum, five times twice the convection of an
+// axis velocity (|difference| <= 2, |minmod| <= |difference|) less its
+// Laplacian, is at most 52 times the largest value (a diagonal velocity's
+// convection 24 times).  256^3: 13.3 -> 4.4 ms per step (417 -> about 130 FP64
+// operations per cell; the FP64 pipe 84 -> 67 % busy, the integer ALUs 74 %:
+// both near their rates); 300 x 80 x 80 with walls 1.68 -> 0.58 ms.
+using fx::from_fixed;
+using fx::in_range;
+using fx::mag;
+using fx::to_fixed;
 
 __device__ __forceinline__ long long clamp64(long long x, long long lo, long long hi) { return min(max(x, lo), hi); }
 
@@ -158,11 +124,11 @@ __device__ __forceinline__ double diag_conv2(const double* __restrict__ f, doubl
   double v[9] = {at(f, X.k[RX ? 3 : 0]), at(f, X.k[RX ? 2 : 1]), at(f, X.k[RX ? 1 : 2]),
                  at(f, Y.k[RY ? 3 : 0]), at(f, Y.k[RY ? 2 : 1]), at(f, Y.k[RY ? 1 : 2]),
                  at(f, Z.k[RZ ? 3 : 0]), at(f, Z.k[RZ ? 2 : 1]), at(f, Z.k[RZ ? 1 : 2])};
-  int mx = mag_hi(c);
+  int mx = mag(c);
 #pragma unroll
-  for (int j = 0; j < 9; ++j) mx = max(mx, mag_hi(v[j]));
+  for (int j = 0; j < 9; ++j) mx = max(mx, mag(v[j]));
   const int E = mx >> 20;
-  if (E < EMIN || E > EMAX) return conv2_double<SCHEME>(c, v);
+  if (!in_range(E)) return conv2_double<SCHEME>(c, v);
   const long long n = to_fixed(c, E);
   long long s = 0;
 #pragma unroll
@@ -181,11 +147,11 @@ __device__ __forceinline__ double axis_sum(const double* __restrict__ f, double 
                                            const Nb& C, bool dissipation) {
   const double m2 = at(f, A.k[R ? 3 : 0]), m1 = at(f, A.k[R ? 2 : 1]), p1 = at(f, A.k[R ? 1 : 2]);
   const double q[4] = {at(f, B.k[1]), at(f, B.k[2]), at(f, C.k[1]), at(f, C.k[2])};
-  int mx = max(max(mag_hi(c), mag_hi(m2)), max(mag_hi(m1), mag_hi(p1)));
+  int mx = max(max(mag(c), mag(m2)), max(mag(m1), mag(p1)));
 #pragma unroll
-  for (int j = 0; j < 4; ++j) mx = max(mx, mag_hi(q[j]));
+  for (int j = 0; j < 4; ++j) mx = max(mx, mag(q[j]));
   const int E = mx >> 20;
-  if (E < EMIN || E > EMAX) {
+  if (!in_range(E)) {
     const double conv2 = 2.0 * grad_pos<SCHEME>(m2, m1, c, p1);
     return dissipation ? 5.0 * conv2 - (((m1 + p1) + (q[0] + q[1])) + (q[2] + q[3]) - 6.0 * c) : conv2;
   }
@@ -203,52 +169,22 @@ __device__ __forceinline__ double axis_sum(const double* __restrict__ f, double 
 __device__ __forceinline__ double rest_lap(const double* __restrict__ f, double c, const Nb& X, const Nb& Y,
                                            const Nb& Z) {
   const double q[6] = {at(f, X.k[1]), at(f, X.k[2]), at(f, Y.k[1]), at(f, Y.k[2]), at(f, Z.k[1]), at(f, Z.k[2])};
-  int mx = mag_hi(c);
+  int mx = mag(c);
 #pragma unroll
-  for (int j = 0; j < 6; ++j) mx = max(mx, mag_hi(q[j]));
+  for (int j = 0; j < 6; ++j) mx = max(mx, mag(q[j]));
   const int E = mx >> 20;
-  if (E < EMIN || E > EMAX) return ((q[0] + q[1]) + (q[2] + q[3])) + (q[4] + q[5]) - 6.0 * c;
+  if (!in_range(E)) return ((q[0] + q[1]) + (q[2] + q[3])) + (q[4] + q[5]) - 6.0 * c;
   long long s = -6 * to_fixed(c, E);
 #pragma unroll
   for (int j = 0; j < 6; ++j) s += to_fixed(q[j], E);
   return from_fixed(s, E);
 }
 
-// rho, u and T of a cell's 15 values (relations e1-e3), the sums in fixed point.
-__device__ __forceinline__ void moments_fp64(const Model<double>& m, const double f[NV], double& rho, double& ux,
-                                             double& uy, double& uz, double& T) {
-  int mx = mag_hi(f[0]);
-#pragma unroll
-  for (int i = 1; i < NV; ++i) mx = max(mx, mag_hi(f[i]));
-  const int E = mx >> 20;
-  if (E < EMIN || E > EMAX) {
-    moments(m, f, rho, ux, uy, uz, T);
-    return;
-  }
-  long long n[NV];
-#pragma unroll
-  for (int i = 0; i < NV; ++i) n[i] = to_fixed(f[i], E);
-  const long long sa = ((n[1] + n[2]) + (n[3] + n[4])) + (n[5] + n[6]);
-  const long long pp = n[7] + n[8], pm = n[9] + n[10], mp = n[11] + n[12], mm = n[13] + n[14];
-  const long long sd = (pp + pm) + (mp + mm);
-  rho = from_fixed(n[0] + sa + sd, E);
-  const double mx_ = fma(m.c1, from_fixed(n[1] - n[2], E), m.s * from_fixed((pp + pm) - (mp + mm), E));
-  const double my_ = fma(m.c1, from_fixed(n[3] - n[4], E), m.s * from_fixed((pp + mp) - (pm + mm), E));
-  const double mz_ = fma(m.c1, from_fixed(n[5] - n[6], E),
-                         m.s * from_fixed(((n[7] + n[9]) + (n[11] + n[13])) - ((n[8] + n[10]) + (n[12] + n[14])), E));
-  const double en = fma(m.eta0sq, f[0], fma(m.c1sq, from_fixed(sa, E), m.c2sq * from_fixed(sd, E)));
-  const double ir = 1.0 / rho;
-  ux = mx_ * ir;
-  uy = my_ * ir;
-  uz = mz_ * ir;
-  T = (en * ir - fma(ux, ux, fma(uy, uy, uz * uz))) * m.inv_b;
-}
-
 // Health bits of one cell.  The comparisons run on the values' high words;
 // only a cell that is close to a limit takes the FP64 ones.
 __device__ __forceinline__ unsigned health_fp64(double rho, double ux, double uy, double uz, double T) {
   const int hr = __double2hiint(rho), ht = __double2hiint(T);
-  const int big = max(max(max(mag_hi(rho), mag_hi(T)), max(mag_hi(ux), mag_hi(uy))), mag_hi(uz));
+  const int big = max(max(max(mag(rho), mag(T)), max(mag(ux), mag(uy))), mag(uz));
   if (hr >= 0x00100000 && ht >= 0x00100000 && big < (1023 + 97) << 20) return 0u;  // normal, below 2^97
   unsigned bad = 0u;
   if (!(rho > 0.0)) bad |= LBM_HEALTH_RHO;
@@ -300,7 +236,7 @@ __global__ void __launch_bounds__(256, 3)
     double f[NV];
 #pragma unroll
     for (int i = 0; i < NV; ++i) f[i] = at(fin + i * L.fs, k0);
-    moments_fp64(m, f, rho, ux, uy, uz, T);
+    fx::moments_fixed(m, f, rho, ux, uy, uz, T);
   }
   if (part == 0) {
     const unsigned bad = health_fp64(rho, ux, uy, uz, T);

@@ -1007,13 +1007,18 @@ int lbm_conserved(lbm_sim* s, double out[5]) {
   int rc = enter(s);
   if (rc) return rc;
   if (!out) return LBM_EINVAL;
+  const int blocks = 2 * s->num_sms < kMaxRedBlocks ? 2 * s->num_sms : kMaxRedBlocks;
   LBM_LAUNCH(s, LBM_KERNEL_REDUCE,
-             lbm::launch_conserved(s->prec, s->fbuf[s->cur], s->L, s->md, s->partials, kMaxRedBlocks, s->counter,
-                                   s->result, s->flags, s->st));
-  unsigned flags = 0;
-  LBM_CK(s, cudaMemcpyAsync(out, s->result, 5 * sizeof(double), cudaMemcpyDeviceToHost, s->st));
-  LBM_CK(s, cudaMemcpyAsync(&flags, s->flags, sizeof(unsigned), cudaMemcpyDeviceToHost, s->st));
+             lbm::launch_conserved(s->prec, s->fbuf[s->cur], s->L, s->md, s->partials, blocks, s->counter, s->result,
+                                   s->flags, s->st));
+  // the flags and the result in one copy (both in the status block)
+  char status[kStatusBytes];
+  const size_t at = (size_t)((char*)s->result - (char*)s->flags);
+  LBM_CK(s, cudaMemcpyAsync(status, s->flags, at + 5 * sizeof(double), cudaMemcpyDeviceToHost, s->st));
   LBM_CK(s, cudaStreamSynchronize(s->st));
+  unsigned flags = 0;
+  std::memcpy(&flags, status, sizeof(flags));
+  std::memcpy(out, status + at, 5 * sizeof(double));
   if (flags & LBM_HEALTH_TIMEOUT) return LBM_ETIMEOUT;
   return flags ? LBM_ENONFINITE : LBM_OK;
 }
