@@ -15,15 +15,24 @@
 // radius max |omega| over a batch of states, wave-vector directions and
 // wave numbers k dx = pi q / nk (q = 1 .. nk): the paper's stability measure.
 //
-// One thread per matrix.  The eigenvalues come from a Householder reduction
-// to upper Hessenberg form followed by the single-shift complex QR
-// iteration with Wilkinson shifts, deflation at negligible subdiagonal
-// entries and an exceptional shift after 10 and 20 iterations without one
-// (the practical QR algorithm of Golub and Van Loan, Sec. 7.5, here without
-// accumulating the transformations: only eigenvalues are needed, so each QR
-// step acts on the unreduced diagonal block alone).  A matrix that has not
-// converged after 30 n iterations reports +inf, which the caller reads as
-// unstable.  The matrices live in shared memory, interleaved by thread.
+// The eigenvalues come from a Householder reduction to upper Hessenberg form
+// followed by the single-shift complex QR iteration with Wilkinson shifts,
+// deflation at negligible subdiagonal entries and an exceptional shift after
+// 10 and 20 iterations without one (the practical QR algorithm of Golub and
+// Van Loan, Sec. 7.5, here without accumulating the transformations: only
+// eigenvalues are needed, so each QR step acts on the unreduced diagonal block
+// alone).  A matrix that has not converged after 30 n iterations reports +inf,
+// which the caller reads as unstable.
+//
+// Bound by the FP64 pipe and, with few matrices per SM, by its latency: a
+// request's 5760 matrices were 180 warps at one thread per matrix, about one
+// per SM, each in a serial chain of FP64 operations (5.05 ms; now 1.72, the
+// FP64 pipe 75 % busy).
+// VT lanes share a matrix: they own columns in the transformations from the
+// left, rows in those from the right, and repeat the scalar work (shifts,
+// rotations) between them, with a synchronisation of the VT lanes at each
+// rotation.  The matrices live in shared memory, VSTRIDE elements apart, so
+// that the two matrices of a quarter warp use different banks.
 #include <cmath>
 
 #include "lbm_internal.cuh"
@@ -32,7 +41,8 @@ namespace lbm {
 namespace {
 
 constexpr int VN = NV;              // matrix order
-constexpr int VN_THREADS = 32;      // matrices per block
+constexpr int VN_THREADS = 32;      // one warp per block
+constexpr int VSTRIDE = VN * VN + 3;  // elements between matrices
 constexpr int VN_PARAMS = 7;        // c1, c2, eta0, gamma, dt, tau, dx
 constexpr int VN_MAX_ITER = 30 * VN;
 
@@ -45,12 +55,16 @@ __device__ __forceinline__ cd operator-(cd a, cd b) { return {a.re - b.re, a.im 
 __device__ __forceinline__ cd operator*(cd a, cd b) { return {a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re}; }
 __device__ __forceinline__ cd operator*(double s, cd a) { return {s * a.re, s * a.im}; }
 __device__ __forceinline__ cd cconj(cd a) { return {a.re, -a.im}; }
+__device__ __forceinline__ double norm2(cd a) { return fma(a.re, a.re, a.im * a.im); }
 __device__ __forceinline__ double cabs(cd a) { return hypot(a.re, a.im); }
-__device__ __forceinline__ double cabs1(cd a) { return fabs(a.re) + fabs(a.im); }
-__device__ __forceinline__ cd cdiv(cd a, cd b) {
-  const double d = b.re * b.re + b.im * b.im;
-  return {(a.re * b.re + a.im * b.im) / d, (a.im * b.re - a.re * b.im) / d};
+// acc + a b and acc - a b
+__device__ __forceinline__ cd fmadd(cd a, cd b, cd acc) {
+  return {fma(a.re, b.re, fma(-a.im, b.im, acc.re)), fma(a.re, b.im, fma(a.im, b.re, acc.im))};
 }
+__device__ __forceinline__ cd fmsub(cd a, cd b, cd acc) {
+  return {fma(-a.re, b.re, fma(a.im, b.im, acc.re)), fma(-a.re, b.im, fma(-a.im, b.re, acc.im))};
+}
+__device__ __forceinline__ double cabs1(cd a) { return fabs(a.re) + fabs(a.im); }
 __device__ __forceinline__ cd csqrt_(cd a) {
   const double r = cabs(a);
   if (r == 0.0) return {0.0, 0.0};
@@ -58,10 +72,27 @@ __device__ __forceinline__ cd csqrt_(cd a) {
   return a.re >= 0.0 ? cd{t, a.im / (2.0 * t)} : cd{fabs(a.im) / (2.0 * t), copysign(t, a.im)};
 }
 
-// Matrix of this thread: element (r, c) at m[(r * VN + c) * VN_THREADS].
+// Matrix of this thread's group of VT lanes (4 or 8), row-major; g is the thread's place
+// in the group, mask the group's lanes of the warp.
+template <int VT_>
 struct Mat {
+  static constexpr int VT = VT_;
   cd* m;
-  __device__ cd& at(int r, int c) const { return m[(r * VN + c) * VN_THREADS]; }
+  int g;
+  unsigned mask;
+  __device__ cd& at(int r, int c) const { return m[r * VN + c]; }
+  __device__ void sync() const { __syncwarp(mask); }
+  // sum and maximum over the group, the same value in every lane
+  __device__ double sum(double v) const {
+#pragma unroll
+    for (int o = VT / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
+    return v;
+  }
+  __device__ double max(double v) const {
+#pragma unroll
+    for (int o = VT / 2; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(mask, v, o));
+    return v;
+  }
 };
 
 // The discrete velocities (Sec. 2) in the library's order: 0 rest; 1..6 +-c1
@@ -96,87 +127,98 @@ __device__ void shell(int i, double c1, double c2, double eta0, double b, double
   }
 }
 
-// G(k) of the state st = (rho, u1, u2, u3, T) and parameters p into M.
+// G(k) of the state st = (rho, u1, u2, u3, T) and parameters p into M; each
+// lane writes rows g, g + VT, ...
+template <class Mat>
 __device__ void build_g(const Mat& M, const double* st, const double* p, const double kv[3], int dissipation) {
+  constexpr int VT = Mat::VT;
   const double c1 = p[0], c2 = p[1], eta0 = p[2], gamma = p[3], dt = p[4], tau = p[5], dx = p[6];
   const double b = 2.0 / (gamma - 1.0), s = c2 / sqrt(3.0);
   const double rho = st[0], u[3] = {st[1], st[2], st[3]}, T = st[4];
   const double usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-  const double r = dt / tau;
-  // column factors of the chain rule: d u_a/df_j and d T/df_j
-  double du[VN][3], dT[VN];
-  for (int j = 0; j < VN; ++j) {
-    double vj[3];
-    velocity(j, c1, s, vj);
-    double rel2 = 0.0;
-    for (int a = 0; a < 3; ++a) {
-      du[j][a] = (vj[a] - u[a]) / rho;
-      rel2 += (vj[a] - u[a]) * (vj[a] - u[a]);
-    }
-    const double eta = j == 0 ? eta0 : 0.0;
-    dT[j] = (rel2 + eta * eta - b * T) / (b * rho);
-  }
-  for (int i = 0; i < VN; ++i) {
+  const double r = dt / tau, ir = 1.0 / rho, ibr = 1.0 / (b * rho);
+  double cs[3], sn[3];
+  for (int a = 0; a < 3; ++a) sincos(kv[a] * dx, &sn[a], &cs[a]);
+#pragma unroll 1
+  for (int i = M.g; i < VN; i += VT) {
     double vi[3], co[7];
     velocity(i, c1, s, vi);
     shell(i, c1, c2, eta0, b, co);
     const double w = vi[0] * u[0] + vi[1] * u[1] + vi[2] * u[2];
     const double A = co[0] + co[1] * T + co[2] * usq, B = co[3] + co[4] * T + co[5] * usq, D = co[6];
     const double f_rho = A + B * w + D * w * w;
-    const double f_T = rho * (co[1] + co[4] * w);
-    double f_u[3];
-    for (int a = 0; a < 3; ++a) f_u[a] = rho * ((2.0 * co[2] + 2.0 * co[5] * w) * u[a] + (B + 2.0 * D * w) * vi[a]);
+    const double f_T = rho * (co[1] + co[4] * w) * ibr;  // with the factor of d T/df_j
+    double f_u[3];                                       // with the factor of d u/df_j
+    for (int a = 0; a < 3; ++a)
+      f_u[a] = rho * ((2.0 * co[2] + 2.0 * co[5] * w) * u[a] + (B + 2.0 * D * w) * vi[a]) * ir;
+#pragma unroll 1
     for (int j = 0; j < VN; ++j) {
-      const double J = f_rho + f_T * dT[j] + f_u[0] * du[j][0] + f_u[1] * du[j][1] + f_u[2] * du[j][2];
+      // columns of the chain rule: (v_ja - u_a), |v_j - u|^2 + eta_j^2 - b T
+      double vj[3];
+      velocity(j, c1, s, vj);
+      const double d0 = vj[0] - u[0], d1 = vj[1] - u[1], d2 = vj[2] - u[2];
+      const double e = fma(d0, d0, fma(d1, d1, d2 * d2)) + ((j == 0 ? eta0 * eta0 : 0.0) - b * T);
+      const double J = fma(f_T, e, fma(f_u[0], d0, fma(f_u[1], d1, fma(f_u[2], d2, f_rho))));
       M.at(i, j) = mk(r * J, 0.0);
     }
     // diagonal: relaxation, convection (first-order upwind phase), dissipation
     const double lam = !dissipation ? 0.0 : (i == 0 ? c1 * dx : (i <= 6 ? c1 * dx / 10.0 : 0.0));
     cd d = mk(1.0 - r, 0.0);
     for (int a = 0; a < 3; ++a) {
-      const double th = kv[a] * dx, cs = cos(th), sn = sin(th);
       // phi = 1 - e^{-i th} = (1 - cos th) + i sin th ; e^{i th} - 1 = (cos th - 1) + i sin th
-      const cd phi = vi[a] >= 0.0 ? mk(1.0 - cs, sn) : mk(cs - 1.0, sn);
+      const cd phi = vi[a] >= 0.0 ? mk(1.0 - cs[a], sn[a]) : mk(cs[a] - 1.0, sn[a]);
       d = d - (vi[a] * dt / dx) * phi;
-      d = d + mk(lam * dt * (2.0 * cs - 2.0) / (dx * dx), 0.0);
+      d = d + mk(lam * dt * (2.0 * cs[a] - 2.0) / (dx * dx), 0.0);
     }
     M.at(i, i) = M.at(i, i) + d;
   }
+  M.sync();
 }
 
-// Spectral radius of M (destroyed), or +inf if the QR iteration does not converge.
-__device__ double spectral_radius(const Mat& M) {
-  const int n = VN;
+// Spectral radius of M (destroyed), or +inf if the QR iteration does not
+// converge; the same value in every lane.  rot: VN rotations of the group.
+struct Rot {
+  cd s;
+  double c;
+};
+template <class Mat>
+__device__ double spectral_radius(const Mat& M, Rot* rot) {
+  constexpr int VT = Mat::VT;
+  const int n = VN, g = M.g;
   // Householder reduction to upper Hessenberg form (similarity, eigenvalues kept)
+#pragma unroll 1
   for (int k = 0; k + 2 < n; ++k) {
-    double tail = 0.0;  // squared norm below the subdiagonal
-    for (int i = k + 2; i < n; ++i) tail += M.at(i, k).re * M.at(i, k).re + M.at(i, k).im * M.at(i, k).im;
+    double part = 0.0;  // squared norm below the subdiagonal
+    for (int i = k + 2 + g; i < n; i += VT) part += norm2(M.at(i, k));
+    const double tail = M.sum(part);
     if (tail == 0.0) continue;  // the column is already in Hessenberg form
-    const double alpha2 = tail + M.at(k + 1, k).re * M.at(k + 1, k).re + M.at(k + 1, k).im * M.at(k + 1, k).im;
-    const double alpha = sqrt(alpha2);
     const cd x0 = M.at(k + 1, k);
-    const double ax0 = cabs(x0);
+    const double p0 = norm2(x0), alpha = sqrt(tail + p0), ax0 = sqrt(p0);
     const cd phase = ax0 > 0.0 ? mk(x0.re / ax0, x0.im / ax0) : mk(1.0, 0.0);
     // v = x + phase alpha e1 (stored in column k below the diagonal), beta = 2 / |v|^2
     const cd v0 = x0 + alpha * phase;
-    M.at(k + 1, k) = v0;
-    const double vn2 = tail + v0.re * v0.re + v0.im * v0.im;
-    const double beta = 2.0 / vn2;
-    for (int j = k + 1; j < n; ++j) {  // left: rows k+1..n-1 of columns k+1..n-1
+    const double beta = 2.0 / (tail + norm2(v0));
+    M.sync();
+    if (g == 0) M.at(k + 1, k) = v0;
+    M.sync();
+    for (int j = k + 1 + g; j < n; j += VT) {  // left: rows k+1..n-1 of columns k+1..n-1
       cd sum = mk(0.0, 0.0);
-      for (int i = k + 1; i < n; ++i) sum = sum + cconj(M.at(i, k)) * M.at(i, j);
+      for (int i = k + 1; i < n; ++i) sum = fmadd(cconj(M.at(i, k)), M.at(i, j), sum);
       sum = beta * sum;
-      for (int i = k + 1; i < n; ++i) M.at(i, j) = M.at(i, j) - M.at(i, k) * sum;
+      for (int i = k + 1; i < n; ++i) M.at(i, j) = fmsub(M.at(i, k), sum, M.at(i, j));
     }
-    for (int r = 0; r < n; ++r) {  // right: columns k+1..n-1 of every row
+    M.sync();
+    for (int r = g; r < n; r += VT) {  // right: columns k+1..n-1 of every row
       cd sum = mk(0.0, 0.0);
-      for (int i = k + 1; i < n; ++i) sum = sum + M.at(r, i) * M.at(i, k);
+      for (int i = k + 1; i < n; ++i) sum = fmadd(M.at(r, i), M.at(i, k), sum);
       sum = beta * sum;
-      for (int i = k + 1; i < n; ++i) M.at(r, i) = M.at(r, i) - sum * cconj(M.at(i, k));
+      for (int i = k + 1; i < n; ++i) M.at(r, i) = fmsub(sum, cconj(M.at(i, k)), M.at(r, i));
     }
+    M.sync();
     // the reflected column: -phase alpha e1
-    M.at(k + 1, k) = (-alpha) * phase;
-    for (int i = k + 2; i < n; ++i) M.at(i, k) = mk(0.0, 0.0);
+    if (g == 0) M.at(k + 1, k) = (-alpha) * phase;
+    for (int i = k + 2 + g; i < n; i += VT) M.at(i, k) = mk(0.0, 0.0);
+    M.sync();
   }
   // shifted QR on the unreduced diagonal blocks, eigenvalues only.  A
   // subdiagonal entry is negligible below ulp times its diagonal neighbours
@@ -185,23 +227,29 @@ __device__ double spectral_radius(const Mat& M) {
   // (those of G for dt = tau are O(Courant number)) is never split off
   const double ulp = 2.220446049250313e-16;
   double nrm = 0.0;
-  for (int r = 0; r < n; ++r)
+  for (int r = g; r < n; r += VT)
     for (int c = r > 0 ? r - 1 : 0; c < n; ++c) nrm = fmax(nrm, cabs1(M.at(r, c)));
-  const double floor_small = ulp * nrm;
+  const double floor_small = ulp * M.max(nrm);
+  const int shift = __ffs((int)M.mask) - 1;
   double radius = 0.0;
   int hi = n - 1, its = 0, total = 0;
-  double gc[VN];
-  cd gs[VN];
+#pragma unroll 1
   while (hi >= 0) {
-    int l = hi;
-    while (l > 0) {
-      const double tst = cabs1(M.at(l - 1, l - 1)) + cabs1(M.at(l, l));
-      if (cabs1(M.at(l, l - 1)) <= fmax(ulp * tst, floor_small)) {
-        M.at(l, l - 1) = mk(0.0, 0.0);
+    int l = 0;  // start of the unreduced block that ends at hi: VT entries are looked at together
+    for (int top = hi; top > 0; top -= VT) {
+      const int i = top - g;
+      bool small = false;
+      if (i > 0) {
+        const double tst = cabs1(M.at(i - 1, i - 1)) + cabs1(M.at(i, i));
+        small = cabs1(M.at(i, i - 1)) <= fmax(ulp * tst, floor_small);
+      }
+      const unsigned found = (__ballot_sync(M.mask, small) >> shift) & ((1u << VT) - 1u);
+      if (found) {
+        l = top - (__ffs((int)found) - 1);
         break;
       }
-      --l;
     }
+    if (l > 0 && g == 0) M.at(l, l - 1) = mk(0.0, 0.0);
     if (l == hi) {  // a 1 x 1 block: an eigenvalue
       const double e = cabs(M.at(hi, hi));
       if (!(e <= 1e300)) return INFINITY;  // non-finite: reported as unstable
@@ -223,39 +271,47 @@ __device__ double spectral_radius(const Mat& M) {
       const cd m1 = d + half + disc, m2 = d + half - disc;
       mu = cabs1(m1 - d) <= cabs1(m2 - d) ? m1 : m2;
     }
-    for (int j = l; j <= hi; ++j) M.at(j, j) = M.at(j, j) - mu;
+    M.sync();
+    for (int j = l + g; j <= hi; j += VT) M.at(j, j) = M.at(j, j) - mu;
+    M.sync();
+#pragma unroll 1
     for (int j = l; j < hi; ++j) {
+      // rotation of rows j, j+1 that takes (x, y) to (|(x, y)|, 0) times x's phase
       const cd x = M.at(j, j), y = M.at(j + 1, j);
-      const double ax = cabs(x), rr = hypot(ax, cabs(y));
-      double cg;
-      cd sg;
-      if (rr == 0.0) {
-        cg = 1.0;
-        sg = mk(0.0, 0.0);
-      } else if (ax == 0.0) {
+      const double px = norm2(x), pn = px + norm2(y);
+      double cg = 1.0;
+      cd sg = mk(0.0, 0.0);
+      if (px >= 1e-280) {
+        const double rs = rsqrt(px * pn);  // 1 / (|x| |(x, y)|)
+        cg = px * rs;
+        sg = rs * (x * cconj(y));
+      } else if (pn >= 1e-280) {  // x = 0 beside y: exchange the rows
         cg = 0.0;
         sg = mk(1.0, 0.0);
-      } else {
-        cg = ax / rr;
-        sg = (1.0 / rr) * (mk(x.re / ax, x.im / ax) * cconj(y));
       }
-      gc[j] = cg;
-      gs[j] = sg;
-      for (int col = j; col <= hi; ++col) {
+      if (g == 0) rot[j] = {sg, cg};
+      M.sync();
+      for (int col = j + g; col <= hi; col += VT) {
         const cd t1 = M.at(j, col), t2 = M.at(j + 1, col);
-        M.at(j, col) = cg * t1 + sg * t2;
-        M.at(j + 1, col) = cg * t2 - cconj(sg) * t1;
+        M.at(j, col) = fmadd(sg, t2, cg * t1);
+        M.at(j + 1, col) = fmsub(cconj(sg), t1, cg * t2);
       }
+      M.sync();
     }
-    for (int j = l; j < hi; ++j) {
-      const int rmax = j + 2 < hi ? j + 2 : hi;
-      for (int r = l; r <= rmax; ++r) {
-        const cd t1 = M.at(r, j), t2 = M.at(r, j + 1);
-        M.at(r, j) = gc[j] * t1 + cconj(gs[j]) * t2;
-        M.at(r, j + 1) = gc[j] * t2 - gs[j] * t1;
+    for (int r = l + g; r <= hi; r += VT) {  // the rows of R times the rotations' adjoints
+      int j = r - 1 > l ? r - 1 : l;
+      cd t1 = M.at(r, j);
+      for (; j < hi; ++j) {
+        const cd t2 = M.at(r, j + 1), sj = rot[j].s;
+        const double cj = rot[j].c;
+        M.at(r, j) = fmadd(cconj(sj), t2, cj * t1);
+        t1 = fmsub(sj, t1, cj * t2);
       }
+      M.at(r, hi) = t1;
     }
-    for (int j = l; j <= hi; ++j) M.at(j, j) = M.at(j, j) + mu;
+    M.sync();
+    for (int j = l + g; j <= hi; j += VT) M.at(j, j) = M.at(j, j) + mu;
+    M.sync();
   }
   return radius;
 }
@@ -263,13 +319,17 @@ __device__ double spectral_radius(const Mat& M) {
 // Item t of the batch: parameter set t / per_param, then state, direction and
 // wave number; out[p] is the max over its items (atomic max of the bit
 // patterns, which order like the values for non-negative doubles).
+template <int VT>
 __global__ void __launch_bounds__(VN_THREADS)
     vn_kernel(const double* __restrict__ states, int nstates, const double* __restrict__ params, int nparams,
               const double* __restrict__ dirs, int ndirs, int nk, int dissipation,
               unsigned long long* __restrict__ out) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int VN_MATS = VN_THREADS / VT;
+  __shared__ __align__(16) cd mats[VN_MATS * VSTRIDE];
+  __shared__ Rot rots[VN_MATS][VN];
   const long long per_param = (long long)nstates * ndirs * nk;
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int slot = threadIdx.x / VT;
+  const long long t = (long long)blockIdx.x * VN_MATS + slot;
   if (t >= per_param * nparams) return;
   const int p = (int)(t / per_param);
   long long rem = t % per_param;
@@ -281,31 +341,31 @@ __global__ void __launch_bounds__(VN_THREADS)
   const double dx = params[VN_PARAMS * p + 6];
   const double kdx = 3.141592653589793 * (q + 1) / nk;
   const double kv[3] = {dv[0] / dn * kdx / dx, dv[1] / dn * kdx / dx, dv[2] / dn * kdx / dx};
-  Mat M{reinterpret_cast<cd*>(smem_raw) + threadIdx.x};
+  Mat<VT> M{mats + slot * VSTRIDE, (int)threadIdx.x % VT, ((1u << VT) - 1u) << (slot * VT)};
   build_g(M, states + 5 * s, params + VN_PARAMS * p, kv, dissipation);
-  const double rad = spectral_radius(M);
-  atomicMax(out + p, (unsigned long long)__double_as_longlong(rad));
+  const double rad = spectral_radius(M, rots[slot]);
+  if (M.g == 0) atomicMax(out + p, (unsigned long long)__double_as_longlong(rad));
 }
-
-constexpr size_t kVnSmem = (size_t)VN * VN * VN_THREADS * sizeof(cd);  // 115,200 bytes
 
 }  // namespace
 
 cudaError_t launch_vn_max_growth(const double* states, int nstates, const double* params, int nparams,
                                  const double* dirs, int ndirs, int nk, int dissipation, double* out,
                                  cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(vn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVnSmem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
   cudaError_t e = cudaMemsetAsync(out, 0, sizeof(double) * nparams, st);
   if (e != cudaSuccess) return e;
+  // Lanes per matrix: with fewer than 16 matrices per SM four lanes leave too
+  // few warps to cover the FP64 pipe's latency, with more eight repeat too much
+  // scalar work (us: 1920 matrices 1448 with four, 1031 with eight; 5760
+  // matrices 1723 and 2050; one lane each 4980 and 5054, two 2378 and 2449).
   const long long items = (long long)nstates * ndirs * nk * nparams;
-  const long long blocks = (items + VN_THREADS - 1) / VN_THREADS;
-  vn_kernel<<<(unsigned)blocks, VN_THREADS, kVnSmem, st>>>(states, nstates, params, nparams, dirs, ndirs, nk,
-                                                           dissipation, reinterpret_cast<unsigned long long*>(out));
+  auto run = [&](auto kernel, int mats) {
+    kernel<<<(unsigned)((items + mats - 1) / mats), VN_THREADS, 0, st>>>(states, nstates, params, nparams, dirs, ndirs, nk,
+                                                                        dissipation,
+                                                                        reinterpret_cast<unsigned long long*>(out));
+  };
+  if (items < 16LL * 152) run(vn_kernel<8>, VN_THREADS / 8);
+  else run(vn_kernel<4>, VN_THREADS / 4);
   return cudaGetLastError();
 }
 
