@@ -85,12 +85,12 @@ enum { LBM_HEALTH_NONFINITE = 1u, LBM_HEALTH_RHO = 2u, LBM_HEALTH_T = 4u, LBM_HE
  * step kernel takes care of periodic axes, reflecting faces and extrapolating
  * x faces itself, so no fill launch is needed between steps (but for odd nx at
  * the x-hi face, odd ny at a reflecting y-hi face, extrapolating y and z faces
- * and FP64 temperature recovery); TILED64 = the same on 64 x 8 tiles (one CTA
- * of 8 warps per SM, run as two halves of 4 warps with their own barriers);
- * TILED_FILL = the TILED kernel with the periodic layers left to a fill launch
- * before each step; TILED_SINGLE = 32 x 8 tiles, one cell per thread; PLAIN =
- * one thread per cell reading global memory; TILED_SPLIT = TILED.  TILED,
- * TILED64, TILED_FILL and TILED_SPLIT give bitwise the same results.
+ * and FP64 temperature recovery); TILED_FILL = the TILED kernel with the
+ * periodic layers left to a fill launch before each step; TILED_SINGLE = 32 x
+ * 8 tiles, one cell per thread; PLAIN = one thread per cell reading global
+ * memory; TILED64 and TILED_SPLIT (once 64 x 8 tiles, and two warp groups per
+ * tile, both slower on every size) = TILED.  TILED, TILED64, TILED_FILL and
+ * TILED_SPLIT give bitwise the same results.
  * lbm_step_batch takes TILED, TILED64 or TILED_SPLIT sims (all the same). */
 enum {
   LBM_VARIANT_TILED = 0,

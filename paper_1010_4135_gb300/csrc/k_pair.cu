@@ -1,12 +1,11 @@
 // Tiled single-precision fused step, two x-adjacent cells per thread.
 //
 // Same plane ring as step_tiled_kernel (one 4D TMA copy per z plane into an
-// mbarrier-tracked ring; see tma_ring.cuh), but each thread of a TX x 8 tile
-// (PairGeo below; 32 x 8 and 128 threads by default) owns the cell pair
-// (x, x+1).  The pair is loaded with one
-// 64-bit shared load per field and neighbour row, and everything that is the
-// same arithmetic for both cells runs as packed f32x2 operations (FADD2,
-// FMUL2, FFMA2), which halves the instructions the schedulers issue.
+// mbarrier-tracked ring; see tma_ring.cuh), but each thread of a 32 x 8 tile
+// owns the cell pair (x, x+1).  The pair is loaded with one 64-bit shared load
+// per field and neighbour row, and everything that is the same arithmetic for
+// both cells runs as packed f32x2 operations (FADD2, FMUL2, FFMA2), which
+// halves the instructions the schedulers issue.
 //
 // Per interface the NND minmod is evaluated once: minmod(x, d) is x clamped
 // to [min(d, 0), max(d, 0)], the two minmods of one cell share d, the pair
@@ -44,20 +43,14 @@ using ring::tma_load_plane;
 // Tile geometry of the pair kernel: a TX x TY column of cells, one thread per
 // cell pair (x, x+1), and a four-plane ring: cell plane z reads ring planes z
 // (its x / y neighbours) and z+1 while z+2 and z+3 land.
-template <int TX_, int TY_, bool SPLIT_ = false>
+template <int TX_, int TY_>
 struct PairGeo {
   static constexpr int TX = TX_, TY = TY_, NSLOT = 4;
-  // SPLIT: the CTA works as two independent halves of 128 threads (the left
-  // and right 32 x 8 cells), each with its own named barrier per plane; a
-  // slot is refilled by whichever half releases it second (release counters
-  // after the mbarriers), so one half can run a plane ahead of the other.
-  static constexpr bool SPLIT = SPLIT_;
   static constexpr int BX = TX + 2 * TMA_LEFT, BY = TY + 4;  // tile with its halo
   static constexpr int PL = BX * BY;                          // floats per field in one plane tile
   static constexpr int SLOT_BYTES = NV * PL * 4;              // bytes one TMA copy delivers
   static constexpr int SLOT_STRIDE = (SLOT_BYTES + 127) / 128 * 128;
-  // slots, then the mbarriers, then (SPLIT) the release counters and the issued-plane count
-  static constexpr int SMEM = NSLOT * SLOT_STRIDE + NSLOT * 8 + (SPLIT ? 64 : 0);
+  static constexpr int SMEM = NSLOT * SLOT_STRIDE + NSLOT * 8;  // slots, then the mbarriers
   static constexpr int PX = TX / 2;                           // threads along x
   static constexpr int THREADS = PX * TY;
   // CTAs per SM that the shared memory allows (228 KB per SM, 1 KB reserved
@@ -69,20 +62,16 @@ struct PairGeo {
                 "64-bit shared loads: a half warp (one 128-byte wavefront) reads one contiguous tile row");
   static_assert(BX * 4 % 16 == 0 && BX <= 256, "TMA box inner extent: a 16-byte multiple, at most 256");
   static_assert(TX % 32 == 0, "tile rows start on 32-byte sectors (OX is a multiple of 8)");
-  static_assert(!SPLIT || (PX == 32 && TY == 8), "split halves: 16 pairs x 8 rows of 128 threads each");
-  // SPLIT: thread t of half h = t / 128 owns pair column 16 h + t % 16 of row (t % 128) / 16
-  __device__ static int col(int tid) { return SPLIT ? (tid & 15) + 16 * (tid >> 7) : tid % PX; }
-  __device__ static int row(int tid) { return SPLIT ? (tid & 127) >> 4 : tid / PX; }
 };
 // 32 x 8 tiles (the single-cell tiled kernel's box, 40 x 12): two CTAs of 4
 // warps per SM.  With two planes in flight an L2 prefetch of later ones only
 // adds L2 lookups (256^3, us per step: 385; one plane ahead 401, two 399,
 // three 410 and more; with one plane in flight it was needed: 475 against 488).
-using Geo32 = PairGeo<ring::TX, ring::TY>;
-// 64 x 8 tiles (box 72 x 12 x 1 x 15): one CTA of 8 warps per SM, 288-byte
-// row reads, run as two split halves: 426 us per step on 256^3.
-using Geo64 = PairGeo<64, 8, true>;
-static_assert(Geo32::BX == ring::BX && Geo32::BY == ring::BY, "Geo32 shares the tiled kernel's tensor map");
+// Larger tiles re-read fewer halo cells, but leave one CTA per SM: 64 x 8 in
+// two halves 426, 32 x 16 415, 32 x 24 and 64 x 12 in three slots with 12
+// warps of 168 registers 437 and 434.
+using Geo = PairGeo<ring::TX, ring::TY>;
+static_assert(Geo::BX == ring::BX && Geo::BY == ring::BY, "Geo shares the tiled kernel's tensor map");
 
 using pm::bc2;
 using pm::ld2;
@@ -103,20 +92,6 @@ struct Opt {
   static constexpr bool FULL = FULL_, R1 = R1_, RD = RD_, XF = XF_, WALL = WALL_, FEW = FEW_;
 };
 
-// Named barrier `id` over 128 threads with an OR of v across them.
-__device__ __forceinline__ bool half_sync_or(unsigned id, bool v) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.ne.u32 p, %1, 0;\n\t"
-      "bar.red.or.pred q, %2, 128, p;\n\t"
-      "selp.u32 %0, 1, 0, q;\n\t}"
-      : "=r"(r)
-      : "r"((unsigned)v), "r"(id)
-      : "memory");
-  return r != 0u;
-}
-
 // One z-march unit: the TX x TY column at (x0, y0), planes z0 .. z0+nzc-1.
 // Plane j of the unit is the ring's plane number jb + j (slot (jb+j) % NSLOT,
 // phase parity ((jb+j) / NSLOT) & 1), so consecutive units of a CTA keep
@@ -131,7 +106,7 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* _
                                           unsigned& jb, bool& timed_out, unsigned wait_limit) {
   constexpr int NSLOT = G::NSLOT, PL = G::PL, BX = G::BX;
   const int tid = threadIdx.x;
-  const int tx = G::col(tid), ty = G::row(tid);
+  const int tx = tid % G::PX, ty = tid / G::PX;
   const int x = x0 + 2 * tx, y = y0 + ty;
   const bool act0 = O::FULL || ((x < L.nx) && (y < L.ny));
   const bool act1 = O::FULL || ((x + 1 < L.nx) && (y < L.ny));
@@ -148,21 +123,16 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* _
   };
 
   // copy ring plane j (interior z0 + j, padded two more) into its slot
-  // (SPLIT: release counters and the count of issued planes follow the mbarriers)
-  unsigned* rel = reinterpret_cast<unsigned*>(bars + NSLOT);
-  int* issued_s = reinterpret_cast<int*>(rel + NSLOT);
-  int issued = 0;  // thread 0 only (without SPLIT)
+  int issued = 0;  // thread 0 only
   auto issue = [&](int j) {
     const unsigned g = jb + (unsigned)j;
     float* dst = reinterpret_cast<float*>(smem + (g % NSLOT) * G::SLOT_STRIDE);
     mbar_expect_tx(&bars[g % NSLOT], G::SLOT_BYTES);
     tma_load_plane(dst, tin, x0 + OX - TMA_LEFT, y0, zplane(z0 + j) + 2, &bars[g % NSLOT]);
-    if (G::SPLIT) atomicMax(issued_s, j + 1);
-    else issued = j + 1;
+    issued = j + 1;
   };
   if (tid == 0) {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    if (G::SPLIT) *issued_s = 0;
     for (int j = 0; j < NSLOT && j < nplanes; ++j) issue(j);
   }
   auto slot = [&](int j) {
@@ -359,35 +329,18 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* _
       F[i] = Z1[i];
     }
     // ring plane k+2 (needed next step) must have landed; the barrier also
-    // marks plane k as retired, so its slot takes plane k + NSLOT
-    const bool ok = arrived(k + 2);
-    if (G::SPLIT) {
-      // this half is done with plane k; the second half to say so refills its slot
-      const unsigned hf = (unsigned)tid >> 7;
-      if (half_sync_or(1u + hf, !ok)) {
-        timed_out = true;
-        break;
-      }
-      if ((tid & 127) == 0) {
-        __threadfence_block();
-        const unsigned prev = atomicAdd(&rel[(jb + (unsigned)k) % NSLOT], 1u);
-        if ((prev & 1u) && k + NSLOT < nplanes) {
-          __threadfence_block();
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          issue(k + NSLOT);
-        }
-      }
-    } else {
-      if (__syncthreads_or(!ok)) {
-        timed_out = true;
-        break;
-      }
-      if (tid == 0 && k + NSLOT < nplanes) {
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        issue(k + NSLOT);
-      }
+    // marks plane k as retired, so its slot takes plane k + NSLOT (releasing
+    // the slots warp by warp, with no barrier, was slower: 390 us against 383)
+    if (__syncthreads_or(!arrived(k + 2))) {
+      timed_out = true;
+      break;
+    }
+    if (tid == 0 && k + NSLOT < nplanes) {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      issue(k + NSLOT);
     }
   }
+
   // the last plane's deferred fields, from ring plane nzc+1 (landed: the last step waited for it)
   if (nzc > 0 && !timed_out) {
     const float* P1 = slot(nzc + 1);
@@ -415,10 +368,6 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* _
     }
     store(out, nzc - 1, true);
   }
-  // SPLIT halves leave the loop on their own (a half that timed out stops
-  // releasing slots, so the other one's waits run out too): rejoin here
-  if (G::SPLIT) timed_out = __syncthreads_or(timed_out) != 0;
-
   if (nzc > 0 && !timed_out) {
     const float mr[2] = {hmin_rho.x, hmin_rho.y}, mt[2] = {hmin_T.x, hmin_T.y}, hs[2] = {hsum.x, hsum.y};
     const bool on[2] = {act0, act1};
@@ -435,8 +384,7 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* _
   if (timed_out) {
     // leave no copy in flight: the newest plane of each slot is waited for (bounded)
     if (tid == 0) {
-      const int n_issued = G::SPLIT ? *issued_s : issued;
-      for (int j = max(0, n_issued - NSLOT); j < n_issued; ++j) drained(j);
+      for (int j = max(0, issued - NSLOT); j < issued; ++j) drained(j);
     }
     __syncthreads();
   }
@@ -453,10 +401,6 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS_PER_SM)
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int s = 0; s < G::NSLOT; ++s) mbar_init(&bars[s], 1);
-    if (G::SPLIT) {
-      unsigned* rel = reinterpret_cast<unsigned*>(bars + G::NSLOT);
-      for (int s = 0; s < G::NSLOT; ++s) rel[s] = 0u;
-    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
@@ -482,10 +426,6 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS_PER_SM)
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int s = 0; s < G::NSLOT; ++s) mbar_init(&bars[s], 1);
-    if (G::SPLIT) {
-      unsigned* rel = reinterpret_cast<unsigned*>(bars + G::NSLOT);
-      for (int s = 0; s < G::NSLOT; ++s) rel[s] = 0u;
-    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
@@ -532,8 +472,8 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS_PER_SM)
 // What the forms go by, over all grids of a launch.
 struct Need {
   bool full = true, r1 = true, rd = false, xf = false, wall = false, few = false;
-  void add(const Layout& L, int tx, int ty, const Model<float>& m, const WtDesc& wt, const RecoverDesc& r) {
-    full = full && L.nx % tx == 0 && L.ny % ty == 0;
+  void add(const Layout& L, const Model<float>& m, const WtDesc& wt, const RecoverDesc& r) {
+    full = full && L.nx % Geo::TX == 0 && L.ny % Geo::TY == 0;
     r1 = r1 && m.dt_tau == 1.0f && m.keep2 == 0.0f;
     rd = rd || r.on;
     xf = xf || wt.xlo || wt.xhi;
@@ -565,93 +505,68 @@ void with_form(const Need& n, F f) {
   f(General());
 }
 
-template <int SCHEME, class G, class... O>
+template <int SCHEME, class... O>
 cudaError_t set_attributes() {
-  const void* fn[] = {(const void*)step_pair_kernel<SCHEME, G, O>..., (const void*)step_pair_batch_kernel<SCHEME, G, O>...};
+  const void* fn[] = {(const void*)step_pair_kernel<SCHEME, Geo, O>..., (const void*)step_pair_batch_kernel<SCHEME, Geo, O>...};
   cudaError_t e = cudaSuccess;
   for (const void* f : fn)
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, Geo::SMEM);
   return e;
 }
 
-template <int SCHEME, class G>
-cudaError_t launch_scheme(const CUtensorMap& map, const float* fin, float* fout, const Layout& L,
-                          const Model<float>& m, const WtDesc& wt, const RecoverDesc& rd, const ZSched& zs,
-                          unsigned* flags, unsigned wait_limit, cudaStream_t st) {
-  dim3 grid((L.nx + G::TX - 1) / G::TX, (L.ny + G::TY - 1) / G::TY, zs.nch);
+template <int SCHEME>
+void launch_scheme(const CUtensorMap& map, const float* fin, float* fout, const Layout& L, const Model<float>& m,
+                   const WtDesc& wt, const RecoverDesc& rd, const ZSched& zs, unsigned* flags, unsigned wait_limit,
+                   cudaStream_t st) {
+  dim3 grid((L.nx + Geo::TX - 1) / Geo::TX, (L.ny + Geo::TY - 1) / Geo::TY, zs.nch);
   Need need;
-  need.add(L, G::TX, G::TY, m, wt, rd);
+  need.add(L, m, wt, rd);
   with_form<SCHEME>(need, [&](auto o) {
-    launch_chained(step_pair_kernel<SCHEME, G, decltype(o)>, grid, G::THREADS, G::SMEM, st, map, fin, fout, L, m, wt, rd,
-                   zs, flags, wait_limit);
+    launch_chained(step_pair_kernel<SCHEME, Geo, decltype(o)>, grid, Geo::THREADS, Geo::SMEM, st, map, fin, fout, L, m, wt,
+                   rd, zs, flags, wait_limit);
   });
-  return cudaGetLastError();
 }
 
-template <class G>
-cudaError_t launch_geo(int scheme, const CUtensorMap& map, const float* fin, float* fout, const Layout& L,
-                       const Model<float>& m, const WtDesc& wt, const RecoverDesc& rd, const ZSched& zs,
-                       unsigned* flags, unsigned wait_limit, cudaStream_t st) {
-  switch (scheme) {
-    case LBM_SCHEME_NND:
-      return launch_scheme<LBM_SCHEME_NND, G>(map, fin, fout, L, m, wt, rd, zs, flags, wait_limit, st);
-    case LBM_SCHEME_UPWIND2:
-      return launch_scheme<LBM_SCHEME_UPWIND2, G>(map, fin, fout, L, m, wt, rd, zs, flags, wait_limit, st);
-    default: return launch_scheme<LBM_SCHEME_UPWIND1, G>(map, fin, fout, L, m, wt, rd, zs, flags, wait_limit, st);
-  }
-}
-
-template <class G>
-cudaError_t prepare_geo() {
-  cudaError_t e = set_attributes<LBM_SCHEME_NND, G, FullPlain, FullFaces, Plain, Faces, Walls, FewRows, General>();
-  if (e == cudaSuccess) e = set_attributes<LBM_SCHEME_UPWIND2, G, General>();
-  if (e == cudaSuccess) e = set_attributes<LBM_SCHEME_UPWIND1, G, General>();
-  return e;
+template <int SCHEME>
+void launch_batch_scheme(const BatchTable& tab, int grid, cudaStream_t st) {
+  Need need;
+  for (int e = 0; e < tab.n; ++e) need.add(tab.item[e].L, tab.item[e].m, tab.item[e].wt, tab.item[e].rd);
+  with_form<SCHEME>(need, [&](auto o) {
+    launch_chained(step_pair_batch_kernel<SCHEME, Geo, decltype(o)>, grid, Geo::THREADS, Geo::SMEM, st, tab);
+  });
 }
 
 }  // namespace
 
 cudaError_t prepare_pair_kernels() {
-  cudaError_t e = prepare_geo<Geo64>();
-  if (e == cudaSuccess) e = prepare_geo<Geo32>();
+  cudaError_t e = set_attributes<LBM_SCHEME_NND, FullPlain, FullFaces, Plain, Faces, Walls, FewRows, General>();
+  if (e == cudaSuccess) e = set_attributes<LBM_SCHEME_UPWIND2, General>();
+  if (e == cudaSuccess) e = set_attributes<LBM_SCHEME_UPWIND1, General>();
   return e;
 }
 
-PairShape pair_shape(int cols) {
-  if (cols == 64) return {Geo64::TX, Geo64::TY, Geo64::BX, Geo64::BY, Geo64::THREADS, Geo64::CTAS_PER_SM};
-  return {Geo32::TX, Geo32::TY, Geo32::BX, Geo32::BY, Geo32::THREADS, Geo32::CTAS_PER_SM};
-}
+PairShape pair_shape() { return {Geo::TX, Geo::TY, Geo::CTAS_PER_SM}; }
 
-template <int SCHEME, class G>
-void launch_batch_scheme(const BatchTable& tab, int grid, cudaStream_t st) {
-  Need need;
-  for (int e = 0; e < tab.n; ++e)
-    need.add(tab.item[e].L, G::TX, G::TY, tab.item[e].m, tab.item[e].wt, tab.item[e].rd);
-  with_form<SCHEME>(need, [&](auto o) {
-    launch_chained(step_pair_batch_kernel<SCHEME, G, decltype(o)>, grid, G::THREADS, G::SMEM, st, tab);
-  });
-}
-
-template <class G>
-void launch_batch_geo(int scheme, const BatchTable& tab, int grid, cudaStream_t st) {
+cudaError_t launch_step_pair_batch(int scheme, const BatchTable& tab, int grid, cudaStream_t st) {
   switch (scheme) {
-    case LBM_SCHEME_NND: return launch_batch_scheme<LBM_SCHEME_NND, G>(tab, grid, st);
-    case LBM_SCHEME_UPWIND2: return launch_batch_scheme<LBM_SCHEME_UPWIND2, G>(tab, grid, st);
-    default: return launch_batch_scheme<LBM_SCHEME_UPWIND1, G>(tab, grid, st);
+    case LBM_SCHEME_NND: launch_batch_scheme<LBM_SCHEME_NND>(tab, grid, st); break;
+    case LBM_SCHEME_UPWIND2: launch_batch_scheme<LBM_SCHEME_UPWIND2>(tab, grid, st); break;
+    default: launch_batch_scheme<LBM_SCHEME_UPWIND1>(tab, grid, st);
   }
-}
-
-cudaError_t launch_step_pair_batch(int cols, int scheme, const BatchTable& tab, int grid, cudaStream_t st) {
-  if (cols == 64) launch_batch_geo<Geo64>(scheme, tab, grid, st);
-  else launch_batch_geo<Geo32>(scheme, tab, grid, st);
   return cudaGetLastError();
 }
 
-cudaError_t launch_step_pair(int cols, int scheme, const CUtensorMap& map, const float* fin, float* fout,
-                             const Layout& L, const Model<float>& m, const WtDesc& wt, const RecoverDesc& rd,
-                             const ZSched& zs, unsigned* flags, unsigned wait_limit, cudaStream_t st) {
-  if (cols == 64) return launch_geo<Geo64>(scheme, map, fin, fout, L, m, wt, rd, zs, flags, wait_limit, st);
-  return launch_geo<Geo32>(scheme, map, fin, fout, L, m, wt, rd, zs, flags, wait_limit, st);
+cudaError_t launch_step_pair(int scheme, const CUtensorMap& map, const float* fin, float* fout, const Layout& L,
+                             const Model<float>& m, const WtDesc& wt, const RecoverDesc& rd, const ZSched& zs,
+                             unsigned* flags, unsigned wait_limit, cudaStream_t st) {
+  switch (scheme) {
+    case LBM_SCHEME_NND: launch_scheme<LBM_SCHEME_NND>(map, fin, fout, L, m, wt, rd, zs, flags, wait_limit, st); break;
+    case LBM_SCHEME_UPWIND2:
+      launch_scheme<LBM_SCHEME_UPWIND2>(map, fin, fout, L, m, wt, rd, zs, flags, wait_limit, st);
+      break;
+    default: launch_scheme<LBM_SCHEME_UPWIND1>(map, fin, fout, L, m, wt, rd, zs, flags, wait_limit, st);
+  }
+  return cudaGetLastError();
 }
 
 // 1/x as the FP32 step kernels form the inverse density (pm::rcp2), two

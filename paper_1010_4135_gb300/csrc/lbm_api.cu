@@ -173,7 +173,6 @@ struct lbm_sim {
   int ztail;            // pair kernels: short chunks of ztail planes end the z range (0 = none)
   int num_sms;
   CUtensorMap tmap[2];  // FP32: TMA descriptors of the two f buffers, box 40 x 12 x 1 x 15 (32 x 8 tiles)
-  CUtensorMap wmap[2];  // the same with box 72 x 12 x 1 x 15 (64 x 8 tiles, variant TILED64)
   lbm::RecoverDesc rd;  // FP64 temperature recovery of the pair kernel
   // launch counting and event-pair timing
   int64_t launches[LBM_NKERNEL];
@@ -301,12 +300,11 @@ bool wt_variant(int variant) {
   return variant == LBM_VARIANT_TILED || variant == LBM_VARIANT_TILED64 || variant == LBM_VARIANT_TILED_SPLIT;
 }
 
-// Variants that run the pair kernel, and its tile width.
+// Variants that run the pair kernel.
 bool pair_variant(int variant) {
   return variant == LBM_VARIANT_TILED || variant == LBM_VARIANT_TILED_FILL || variant == LBM_VARIANT_TILED64 ||
          variant == LBM_VARIANT_TILED_SPLIT;
 }
-int pair_cols(int variant) { return variant == LBM_VARIANT_TILED64 ? 64 : 32; }
 
 // z planes per CTA of the single-cell tiled kernel when none is set: the
 // largest of 32, 24, 16, 12, 8, 6, 4 that still gives two waves of units.
@@ -538,11 +536,8 @@ int lbm_create(const lbm_grid* grid, const lbm_vset* vset, double tau, double dt
     return LBM_ECUDA;
   }
   if (precision == LBM_FP32) {
-    const lbm::PairShape p64 = lbm::pair_shape(64);
     if (!make_tmap(&s->tmap[0], s->fbuf[0], s->L, lbm::tiled_box_x(), lbm::tiled_box_y()) ||
         !make_tmap(&s->tmap[1], s->fbuf[1], s->L, lbm::tiled_box_x(), lbm::tiled_box_y()) ||
-        !make_tmap(&s->wmap[0], s->fbuf[0], s->L, p64.bx, p64.by) ||
-        !make_tmap(&s->wmap[1], s->fbuf[1], s->L, p64.bx, p64.by) ||
         lbm::prepare_tiled_kernels() != cudaSuccess || lbm::prepare_pair_kernels() != cudaSuccess) {
       delete s;
       return LBM_ECUDA;
@@ -632,7 +627,7 @@ int run_steps(lbm_sim* s, int64_t n) {
     if (rc) return rc;
   }
   const bool pair = s->prec == LBM_FP32 && pair_variant(s->variant);
-  const lbm::PairShape shape = lbm::pair_shape(pair_cols(s->variant));
+  const lbm::PairShape shape = lbm::pair_shape();
   unsigned written = 0, own = 0;
   const lbm::WtDesc wt = write_through(s, &written, &own);
   for (int64_t k = 0; k < n; ++k) {
@@ -645,11 +640,10 @@ int run_steps(lbm_sim* s, int64_t n) {
       LBM_LAUNCH(s, LBM_KERNEL_FILL, lbm::launch_fill(s->prec, fin, s->L, s->md, s->mf, s->bc, mask, s->st));
     if (s->prec == LBM_FP32 && s->variant != LBM_VARIANT_PLAIN) {
       if (pair) {
-        const CUtensorMap& map = shape.tx == 64 ? s->wmap[s->cur] : s->tmap[s->cur];
         const lbm::ZSched zs = s->zchunk > 0 ? lbm::make_zsched(s->L.nz, s->zchunk, s->ztail)
                                              : auto_zsched(s->L, s->num_sms, shape);
         LBM_LAUNCH(s, LBM_KERNEL_STEP,
-                   lbm::launch_step_pair(shape.tx, s->scheme, map, (const float*)fin, (float*)fout, s->L, s->mf, wt,
+                   lbm::launch_step_pair(s->scheme, s->tmap[s->cur], (const float*)fin, (float*)fout, s->L, s->mf, wt,
                                          s->rd, zs, s->flags, s->wait_limit, s->st));
       } else {
         const int zc = s->zchunk > 0 ? s->zchunk : auto_zchunk(s->L, s->num_sms);
@@ -704,7 +698,7 @@ int batch_check(lbm_sim* const* sims, int32_t n) {
 // launch of the persistent tile kernel for all sims.
 int run_batch(lbm_sim* const* sims, int32_t n, int64_t steps) {
   lbm_sim* s0 = sims[0];
-  const lbm::PairShape shape = lbm::pair_shape(pair_cols(s0->variant));
+  const lbm::PairShape shape = lbm::pair_shape();
   for (int i = 0; i < n; ++i) {
     int rc = fill_fixed(sims[i]);
     if (rc) return rc;
@@ -728,7 +722,7 @@ int run_batch(lbm_sim* const* sims, int32_t n, int64_t steps) {
         LBM_LAUNCH(s, LBM_KERNEL_FILL,
                    lbm::launch_fill(s->prec, s->fbuf[s->cur], s->L, s->md, s->mf, s->bc, mask, s->st));
       lbm::BatchItem& it = tab.item[i];
-      tab.map[i] = shape.tx == 64 ? s->wmap[s->cur] : s->tmap[s->cur];
+      tab.map[i] = s->tmap[s->cur];
       it.fin = (const float*)s->fbuf[s->cur];
       it.fout = (float*)s->fbuf[s->cur ^ 1];
       it.flags = s->flags;
@@ -750,7 +744,7 @@ int run_batch(lbm_sim* const* sims, int32_t n, int64_t steps) {
     tab.done = s0->done;
     const long long resident = (long long)shape.ctas_per_sm * s0->num_sms;
     const int grid = (int)(units < resident ? units : resident);
-    LBM_LAUNCH(s0, LBM_KERNEL_STEP, lbm::launch_step_pair_batch(shape.tx, s0->scheme, tab, grid, s0->st));
+    LBM_LAUNCH(s0, LBM_KERNEL_STEP, lbm::launch_step_pair_batch(s0->scheme, tab, grid, s0->st));
     for (int i = 0; i < n; ++i) {
       lbm_sim* s = sims[i];
       s->layers_ok[s->cur ^ 1] = 1;

@@ -257,13 +257,12 @@ cudaError_t launch_step_fp64(int scheme, const double* fin, double* fout, const 
                              unsigned per, int num_sms, unsigned* flags, cudaStream_t st);
 cudaError_t launch_step_tiled(int scheme, const CUtensorMap& map, const float* fin, float* fout, const Layout& L,
                               const Model<float>& m, int zc, unsigned* flags, cudaStream_t st);
-// Pair kernel (two cells per thread) on `cols` x 8 tiles: cols = 64 (box
-// 72 x 12, one CTA per SM) or 32 (the tiled kernel's tiles and box 40 x 12,
-// two CTAs per SM).  The map's box must be pair_shape(cols).bx x .by.
+// Pair kernel (two cells per thread): tile, CTAs per SM; its TMA box is the
+// tiled kernel's (tiled_box_x, tiled_box_y).
 struct PairShape {
-  int tx, ty, bx, by, threads, ctas_per_sm;
+  int tx, ty, ctas_per_sm;
 };
-PairShape pair_shape(int cols);
+PairShape pair_shape();
 
 // How the pair kernels split the z range of a tile column into chunks (one
 // chunk = one unit of work, a z-march of one CTA).  With zt = 0 all chunks
@@ -294,8 +293,8 @@ inline ZSched make_zsched(int nz, int zc, int zt) {
   return z;
 }
 
-cudaError_t launch_step_pair(int cols, int scheme, const CUtensorMap& map, const float* fin, float* fout,
-                             const Layout& L, const Model<float>& m, const WtDesc& wt, const RecoverDesc& rd,
+cudaError_t launch_step_pair(int scheme, const CUtensorMap& map, const float* fin, float* fout, const Layout& L,
+                             const Model<float>& m, const WtDesc& wt, const RecoverDesc& rd,
                              const ZSched& zs, unsigned* flags, unsigned wait_limit, cudaStream_t st);
 
 // Descriptor table of a batched step (passed by value as the kernel
@@ -323,8 +322,8 @@ struct BatchTable {
   unsigned long long* queue;  // next unit to take (0 at launch; reset by the last CTA)
   unsigned* done;             // CTAs finished (0 at launch; reset by the last CTA)
 };
-// Batched step over the descriptor table (`cols` x 8 tiles, maps of that box).
-cudaError_t launch_step_pair_batch(int cols, int scheme, const BatchTable& tab, int grid, cudaStream_t st);
+// Batched step over the descriptor table.
+cudaError_t launch_step_pair_batch(int scheme, const BatchTable& tab, int grid, cudaStream_t st);
 // y = 1/x as the FP32 step kernels form the inverse density (device arrays).
 cudaError_t launch_reciprocal_fp32(const float* x, float* y, long long n, cudaStream_t st);
 // Von Neumann service: out[p] = max |omega| of G(k) (Sec. 3) over the states
