@@ -79,9 +79,12 @@ __global__ void __launch_bounds__(256) step_plain_kernel(const float* __restrict
 // a cell's 15 values).  The largest sum, five times twice the convection of an
 // axis velocity (|difference| <= 2, |minmod| <= |difference|) less its
 // Laplacian, is at most 52 times the largest value (a diagonal velocity's
-// convection 24 times).  256^3: 13.3 -> 4.4 ms per step (417 -> about 130 FP64
-// operations per cell; the FP64 pipe 84 -> 67 % busy, the integer ALUs 74 %:
-// both near their rates); 300 x 80 x 80 with walls 1.68 -> 0.58 ms.
+// convection 24 times).  256^3: 13.3 -> 4.3 ms per step (417 -> 112 FP64
+// operations per cell; the FP64 pipe 84 -> 69 % busy, the integer ALUs 74 %:
+// both near their rates); 300 x 80 x 80 with walls 1.68 -> 0.57 ms.
+// Aligning by one multiplication where the values are within 2^4 of each other
+// saves 900 of 3400 ALU instructions, but the cells at shocks and zero
+// crossings send their warps through both forms (64^3 91 -> 104 us): not kept.
 using fx::from_fixed;
 using fx::in_range;
 using fx::mag;
@@ -101,12 +104,12 @@ __device__ __forceinline__ long long grad2(long long m2, long long m1, long long
   return 2 * d + (clamp64(p1 - c, lo, hi) - clamp64(m1 - m2, lo, hi));
 }
 
-// The same in double, for stencils outside the fixed-point range.
+// The same for three axes in double, for stencils outside the fixed-point range.
 template <int SCHEME>
-__device__ __noinline__ double conv2_double(double c, const double* v) {
-  double s = 0.0;
-  for (int a = 0; a < 3; ++a) s += 2.0 * grad_pos<SCHEME>(v[3 * a], v[3 * a + 1], c, v[3 * a + 2]);
-  return s;
+__device__ __noinline__ double conv2_double(double c, double x0, double x1, double x2, double y0, double y1, double y2,
+                                            double z0, double z1, double z2) {
+  return 2.0 * grad_pos<SCHEME>(x0, x1, c, x2) + 2.0 * grad_pos<SCHEME>(y0, y1, c, y2) +
+         2.0 * grad_pos<SCHEME>(z0, z1, c, z2);
 }
 
 // Field offsets (32-bit, modulo 2^32: a field has fewer elements) of a cell's
@@ -116,19 +119,32 @@ struct Nb {
 };
 __device__ __forceinline__ double at(const double* __restrict__ f, unsigned k) { return __ldg(f + k); }
 
-// Twice the convection sum of a diagonal velocity: x, y, z neighbours; sx, sy, sz
-// reverse an axis.
-template <int SCHEME, bool RX, bool RY, bool RZ>
-__device__ __forceinline__ double diag_conv2(const double* __restrict__ f, double c, const Nb& X, const Nb& Y,
-                                             const Nb& Z) {
-  double v[9] = {at(f, X.k[RX ? 3 : 0]), at(f, X.k[RX ? 2 : 1]), at(f, X.k[RX ? 1 : 2]),
-                 at(f, Y.k[RY ? 3 : 0]), at(f, Y.k[RY ? 2 : 1]), at(f, Y.k[RY ? 1 : 2]),
-                 at(f, Z.k[RZ ? 3 : 0]), at(f, Z.k[RZ ? 2 : 1]), at(f, Z.k[RZ ? 1 : 2])};
+// The values a velocity's update reads besides the cell's own, upwind to
+// downwind m2, m1, p1 along each axis of a diagonal velocity; for an axis one
+// m2, m1, p1 along its axis and the four lateral neighbours.  R..: reversed
+// axes (negative components).
+template <bool RX, bool RY, bool RZ>
+__device__ __forceinline__ void diag_load(const double* __restrict__ f, const Nb& X, const Nb& Y, const Nb& Z,
+                                          double v[9]) {
+  v[0] = at(f, X.k[RX ? 3 : 0]); v[1] = at(f, X.k[RX ? 2 : 1]); v[2] = at(f, X.k[RX ? 1 : 2]);
+  v[3] = at(f, Y.k[RY ? 3 : 0]); v[4] = at(f, Y.k[RY ? 2 : 1]); v[5] = at(f, Y.k[RY ? 1 : 2]);
+  v[6] = at(f, Z.k[RZ ? 3 : 0]); v[7] = at(f, Z.k[RZ ? 2 : 1]); v[8] = at(f, Z.k[RZ ? 1 : 2]);
+}
+template <bool R>
+__device__ __forceinline__ void axis_load(const double* __restrict__ f, const Nb& A, const Nb& B, const Nb& C,
+                                          double v[9]) {
+  v[0] = at(f, A.k[R ? 3 : 0]); v[1] = at(f, A.k[R ? 2 : 1]); v[2] = at(f, A.k[R ? 1 : 2]);
+  v[3] = at(f, B.k[1]); v[4] = at(f, B.k[2]); v[5] = at(f, C.k[1]); v[6] = at(f, C.k[2]);
+}
+
+// Twice the convection sum of a diagonal velocity.
+template <int SCHEME>
+__device__ __forceinline__ double diag_conv2(double c, const double v[9]) {
   int mx = mag(c);
 #pragma unroll
   for (int j = 0; j < 9; ++j) mx = max(mx, mag(v[j]));
   const int E = mx >> 20;
-  if (!in_range(E)) return conv2_double<SCHEME>(c, v);
+  if (!in_range(E)) return conv2_double<SCHEME>(c, v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7], v[8]);
   const long long n = to_fixed(c, E);
   long long s = 0;
 #pragma unroll
@@ -137,38 +153,32 @@ __device__ __forceinline__ double diag_conv2(const double* __restrict__ f, doubl
   return from_fixed(s, E);
 }
 
-// Convection and dissipation of an axis velocity along A (R: the negative
-// one); B, C: the other axes.  With the dissipation term lambda_i = c1 dx / 10
-// (Sec. 3), so both terms are one multiple of lambda_i dt/dx^2 = |v| dt/(10
-// dx): returns 5 times twice the convection less the Laplacian, or twice the
-// convection alone when the term is off.
-template <int SCHEME, bool R>
-__device__ __forceinline__ double axis_sum(const double* __restrict__ f, double c, const Nb& A, const Nb& B,
-                                           const Nb& C, bool dissipation) {
-  const double m2 = at(f, A.k[R ? 3 : 0]), m1 = at(f, A.k[R ? 2 : 1]), p1 = at(f, A.k[R ? 1 : 2]);
-  const double q[4] = {at(f, B.k[1]), at(f, B.k[2]), at(f, C.k[1]), at(f, C.k[2])};
-  int mx = max(max(mag(c), mag(m2)), max(mag(m1), mag(p1)));
+// Convection and dissipation of an axis velocity.  With the dissipation term
+// lambda_i = c1 dx / 10 (Sec. 3), so both terms are one multiple of lambda_i
+// dt/dx^2 = |v| dt/(10 dx): returns 5 times twice the convection less the
+// Laplacian, or twice the convection alone when the term is off.
+template <int SCHEME>
+__device__ __forceinline__ double axis_sum(double c, const double v[9], bool dissipation) {
+  int mx = mag(c);
 #pragma unroll
-  for (int j = 0; j < 4; ++j) mx = max(mx, mag(q[j]));
+  for (int j = 0; j < 7; ++j) mx = max(mx, mag(v[j]));
   const int E = mx >> 20;
   if (!in_range(E)) {
-    const double conv2 = 2.0 * grad_pos<SCHEME>(m2, m1, c, p1);
-    return dissipation ? 5.0 * conv2 - (((m1 + p1) + (q[0] + q[1])) + (q[2] + q[3]) - 6.0 * c) : conv2;
+    const double conv2 = 2.0 * grad_pos<SCHEME>(v[0], v[1], c, v[2]);
+    return dissipation ? 5.0 * conv2 - (((v[1] + v[2]) + (v[3] + v[4])) + (v[5] + v[6]) - 6.0 * c) : conv2;
   }
-  const long long n = to_fixed(c, E), n1 = to_fixed(m1, E), n2 = to_fixed(p1, E);
-  long long s = grad2<SCHEME>(to_fixed(m2, E), n1, n, n2);
+  const long long n = to_fixed(c, E), n1 = to_fixed(v[1], E), n2 = to_fixed(v[2], E);
+  long long s = grad2<SCHEME>(to_fixed(v[0], E), n1, n, n2);
   if (dissipation) {
     s = 5 * s + 6 * n - (n1 + n2);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) s -= to_fixed(q[j], E);
+    for (int j = 3; j < 7; ++j) s -= to_fixed(v[j], E);
   }
   return from_fixed(s, E);
 }
 
-// The Laplacian of the rest velocity.
-__device__ __forceinline__ double rest_lap(const double* __restrict__ f, double c, const Nb& X, const Nb& Y,
-                                           const Nb& Z) {
-  const double q[6] = {at(f, X.k[1]), at(f, X.k[2]), at(f, Y.k[1]), at(f, Y.k[2]), at(f, Z.k[1]), at(f, Z.k[2])};
+// The Laplacian of the rest velocity from its six neighbours.
+__device__ __forceinline__ double rest_lap(double c, const double q[6]) {
   int mx = mag(c);
 #pragma unroll
   for (int j = 0; j < 6; ++j) mx = max(mx, mag(q[j]));
@@ -212,10 +222,9 @@ __device__ __forceinline__ Nb neighbours(int i, int n, bool periodic, unsigned k
 // R1: dt = tau.  The velocities come in opposite pairs that share the even
 // part of f^eq: three axis pairs and four diagonal ones, each a loop whose
 // body serves all of its kind (the neighbour offsets and velocity components
-// take turns), so the code stays short.  `parts` blocks share a row: 1; 3
-// (rest and axis pairs; two diagonal pairs each); or 7 (one pair each, the
-// first with the rest velocity), each with the moments for itself.  kax, kdg:
-// factors of axis_sum and diag_conv2.
+// take turns), so the code stays short.  `parts` blocks share a row: 1, or 3
+// (rest and axis pairs; two diagonal pairs each), each with the moments for
+// itself.  kax, kdg: factors of axis_sum and diag_conv2.
 template <int SCHEME, bool R1>
 __global__ void __launch_bounds__(256, 3)
     step_fp64_kernel(const double* __restrict__ fin, double* __restrict__ fout, Layout L, Model<double> m, double kax,
@@ -223,10 +232,9 @@ __global__ void __launch_bounds__(256, 3)
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = (blockIdx.y / parts) * blockDim.y + threadIdx.y;
   const int z = blockIdx.z, part = blockIdx.y % parts;
-  // the axis pairs [a0, a1) and diagonal pairs [d0, d1) of this part
-  const int a0 = parts == 7 ? part : 0, a1 = parts == 1 ? 3 : (parts == 3 ? (part == 0 ? 3 : 0) : (part < 3 ? part + 1 : 0));
-  const int d0 = parts == 1 ? 0 : (parts == 3 ? 2 * part - 2 : part - 3);
-  const int d1 = parts == 1 ? 4 : (parts == 3 ? 2 * part : part - 2);
+  // the axis pairs [0, a1) and diagonal pairs [d0, d1) of this part
+  const int a1 = part == 0 ? 3 : 0;
+  const int d0 = parts == 1 ? 0 : 2 * part - 2, d1 = parts == 1 ? 4 : 2 * part;
   chain_wait();
   if (x >= L.nx || y >= L.ny) return;
   const unsigned k0 = (unsigned)L.at(x, y, z);
@@ -251,7 +259,8 @@ __global__ void __launch_bounds__(256, 3)
   if (part == 0) {
     const double c = at(fin, k0);
     const double fe = rho * (m.AR * T);
-    fout[k0] = fma(m.lam0, rest_lap(fin, c, X, Y, Z), relax(fe, c));
+    const double q[6] = {at(fin, X.k[1]), at(fin, X.k[2]), at(fin, Y.k[1]), at(fin, Y.k[2]), at(fin, Z.k[1]), at(fin, Z.k[2])};
+    fout[k0] = fma(m.lam0, rest_lap(c, q), relax(fe, c));
   }
   const double usq = fma(ux, ux, fma(uy, uy, uz * uz));
   {
@@ -263,16 +272,17 @@ __global__ void __launch_bounds__(256, 3)
     double ua = ux, ub = uy, uc = uz;
 #pragma unroll 1
     for (int a = 0; a < a1; ++a) {
-      if (a >= a0) {
-        const double w = m.c1 * ua, q = fma(rD, w * w, rA);
-        const double* fp = fin + (1 + 2 * a) * L.fs;
-        double* op = fout + (1 + 2 * a) * L.fs + k0;
-        double c = at(fp, k0);
-        *op = fma(kax, axis_sum<SCHEME, false>(fp, c, A, B, C, dissipation), relax(fma(rB, w, q), c));
-        fp += L.fs;
-        c = at(fp, k0);
-        op[L.fs] = fma(kax, axis_sum<SCHEME, true>(fp, c, A, B, C, dissipation), relax(fma(-rB, w, q), c));
-      }
+      const double w = m.c1 * ua, q = fma(rD, w * w, rA);
+      const double* fp = fin + (1 + 2 * a) * L.fs;
+      double* op = fout + (1 + 2 * a) * L.fs + k0;
+      double v[9];
+      double c = at(fp, k0);
+      axis_load<false>(fp, A, B, C, v);
+      *op = fma(kax, axis_sum<SCHEME>(c, v, dissipation), relax(fma(rB, w, q), c));
+      fp += L.fs;
+      c = at(fp, k0);
+      axis_load<true>(fp, A, B, C, v);
+      op[L.fs] = fma(kax, axis_sum<SCHEME>(c, v, dissipation), relax(fma(-rB, w, q), c));
       const Nb t = A;
       A = B;
       B = C;
@@ -295,13 +305,14 @@ __global__ void __launch_bounds__(256, 3)
       if (k >= d0) {
         const double w = m.s * (uxy + uc), q = fma(rD, w * w, rA);
         const double* fp = fin + (7 + k) * L.fs;
+        double v[9];
         double c = at(fp, k0);
-        fout[(7 + k) * L.fs + k0] =
-            fma(kdg, diag_conv2<SCHEME, false, false, false>(fp, c, X, B, C), relax(fma(rB, w, q), c));
+        diag_load<false, false, false>(fp, X, B, C, v);
+        fout[(7 + k) * L.fs + k0] = fma(kdg, diag_conv2<SCHEME>(c, v), relax(fma(rB, w, q), c));
         fp = fin + (14 - k) * L.fs;
         c = at(fp, k0);
-        fout[(14 - k) * L.fs + k0] =
-            fma(kdg, diag_conv2<SCHEME, true, true, true>(fp, c, X, B, C), relax(fma(-rB, w, q), c));
+        diag_load<true, true, true>(fp, X, B, C, v);
+        fout[(14 - k) * L.fs + k0] = fma(kdg, diag_conv2<SCHEME>(c, v), relax(fma(-rB, w, q), c));
       }
       // reverse z; after the second pair y as well
       auto reverse = [](Nb& n) {
@@ -322,13 +333,89 @@ __global__ void __launch_bounds__(256, 3)
   chain_start();  // late: started early, the next step's blocks gather on the SMs that happen to have room
 }
 
+// The same with one pair of velocities per block (seven parts) and all loads
+// issued before the moments' arithmetic: on a grid of a few hundred rows the
+// step is one warp's latency, and the stencils' loads after the moments were a
+// second trip to the L2 (150 x 1 x 1: 5.2 -> 4.3 us per step, 200 x 4 x 4: 6.3
+// -> 5.9).
+template <int SCHEME, bool R1>
+__global__ void __launch_bounds__(32)
+    step_fp64_pairs_kernel(const double* __restrict__ fin, double* __restrict__ fout, Layout L, Model<double> m,
+                           double kax, double kdg, unsigned per, unsigned* __restrict__ flags) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  const int y = blockIdx.y / 7, z = blockIdx.z, part = blockIdx.y % 7;
+  const bool diag = part >= 3;
+  const int ia = diag ? 4 + part : 1 + 2 * part, ib = diag ? 17 - part : 2 + 2 * part;  // the pair's velocities
+  const unsigned k0 = (unsigned)L.at(x, y, z);
+  const Nb X = neighbours(x, L.nx, per & 1u, k0, 1u), Y = neighbours(y, L.ny, per & 2u, k0, (unsigned)L.sx),
+           Z = neighbours(z, L.nz, per & 4u, k0, (unsigned)L.plane);
+  chain_wait();
+  if (x >= L.nx) return;
+  double f[NV], va[9], vb[9], r6[6];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) f[i] = at(fin + i * L.fs, k0);
+  const double *fa = fin + ia * L.fs, *fb = fin + ib * L.fs;
+  if (diag) {
+    const bool ry = part >= 5, rz = (part & 1) == 0;  // pairs (+,+,+), (+,+,-), (+,-,+), (+,-,-)
+    const Nb B = {{Y.k[ry ? 3 : 0], Y.k[ry ? 2 : 1], Y.k[ry ? 1 : 2], Y.k[ry ? 0 : 3]}};
+    const Nb C = {{Z.k[rz ? 3 : 0], Z.k[rz ? 2 : 1], Z.k[rz ? 1 : 2], Z.k[rz ? 0 : 3]}};
+    diag_load<false, false, false>(fa, X, B, C, va);
+    diag_load<true, true, true>(fb, X, B, C, vb);
+  } else {
+    const Nb A = part == 0 ? X : (part == 1 ? Y : Z), B = part == 0 ? Y : (part == 1 ? Z : X),
+             C = part == 0 ? Z : (part == 1 ? X : Y);
+    axis_load<false>(fa, A, B, C, va);
+    axis_load<true>(fb, A, B, C, vb);
+  }
+  if (part == 0) {
+    const Nb N[3] = {X, Y, Z};
+#pragma unroll
+    for (int j = 0; j < 6; ++j) r6[j] = at(fin, N[j / 2].k[1 + j % 2]);
+  }
+  const double ca = at(fa, k0), cb = at(fb, k0);
+
+  double rho, ux, uy, uz, T;
+  fx::moments_fixed(m, f, rho, ux, uy, uz, T);
+  auto relax = [&](double fe, double fc) { return R1 ? fe : fma(m.keep2, fc, m.dt_tau * fe); };
+  if (part == 0) {
+    const unsigned bad = health_fp64(rho, ux, uy, uz, T);
+    if (bad) atomicOr(flags, bad);
+    fout[k0] = fma(m.lam0, rest_lap(f[0], r6), relax(rho * (m.AR * T), f[0]));
+  }
+  const double usq = fma(ux, ux, fma(uy, uy, uz * uz));
+  double w, q, rB, ka, sa, sb;
+  if (diag) {
+    const double sy = part >= 5 ? ux - uy : ux + uy;
+    w = m.s * ((part & 1) == 0 ? sy - uz : sy + uz);
+    rB = rho * fma(m.BdT, T, fma(m.BdU, usq, m.Bd0));
+    q = fma(rho * m.Dd, w * w, rho * fma(m.AdT, T, fma(m.AdU, usq, m.Ad0)));
+    ka = kdg;
+    sa = diag_conv2<SCHEME>(ca, va);
+    sb = diag_conv2<SCHEME>(cb, vb);
+  } else {
+    w = m.c1 * (part == 0 ? ux : (part == 1 ? uy : uz));
+    rB = rho * fma(m.BaT, T, fma(m.BaU, usq, m.Ba0));
+    q = fma(rho * m.Da, w * w, rho * fma(m.AaT, T, fma(m.AaU, usq, m.Aa0)));
+    ka = kax;
+    sa = axis_sum<SCHEME>(ca, va, m.lam1 != 0.0);
+    sb = axis_sum<SCHEME>(cb, vb, m.lam1 != 0.0);
+  }
+  fout[ia * L.fs + k0] = fma(ka, sa, relax(fma(rB, w, q), ca));
+  fout[ib * L.fs + k0] = fma(ka, sb, relax(fma(-rB, w, q), cb));
+  chain_start();
+}
+
 template <int SCHEME>
 void launch_fp64(const double* fin, double* fout, const Layout& L, const Model<double>& m,
                  unsigned per, int parts, dim3 grid, dim3 block, unsigned* flags,
                  cudaStream_t st) {
   const double kax = m.lam1 != 0.0 ? -0.1 * m.k1 : -0.5 * m.k1;
-  launch_chained(m.dt_tau == 1.0 ? step_fp64_kernel<SCHEME, true> : step_fp64_kernel<SCHEME, false>, grid, block, 0, st,
-                 fin, fout, L, m, kax, -0.5 * m.k2, per, parts, flags);
+  if (parts == 7)
+    launch_chained(m.dt_tau == 1.0 ? step_fp64_pairs_kernel<SCHEME, true> : step_fp64_pairs_kernel<SCHEME, false>, grid,
+                   block, 0, st, fin, fout, L, m, kax, -0.5 * m.k2, per, flags);
+  else
+    launch_chained(m.dt_tau == 1.0 ? step_fp64_kernel<SCHEME, true> : step_fp64_kernel<SCHEME, false>, grid, block, 0, st,
+                   fin, fout, L, m, kax, -0.5 * m.k2, per, parts, flags);
 }
 
 }  // namespace
@@ -352,9 +439,9 @@ cudaError_t launch_step_fp64(int scheme, const double* fin, double* fout, const 
   // all SMs (4000 x 4 x 4, 13 warps per SM: 24 us against 30; from 21 warps per
   // SM on no difference).  Smaller still, a row's 5400 instructions in one warp
   // are the step's length, and its velocities go to several blocks (us per
-  // step with 1 / 3 / 7 parts: 200 x 4 x 4, 0.7 warps per SM, 14.9 / 8.2 / 6.3;
-  // 400 x 4 x 4, 1.4: 14.4 / 8.5 / 7.7; 800 x 4 x 4, 2.6: 14.5 / 10.0 / 11.6;
-  // 2000 x 4 x 4, 6.6: 16.3 / 16.3 / 24.9).
+  // step with 1 / 3 / 7 parts: 200 x 4 x 4, 0.7 warps per SM, 14.9 / 8.2 / 5.9;
+  // 400 x 4 x 4, 1.4: 14.4 / 8.5 / 7.6; 800 x 4 x 4, 2.6: 14.5 / 10.0 / 12.5;
+  // 2000 x 4 x 4, 6.6: 16.3 / 16.1 / 24.7).
   const long long warps = (long long)((L.nx + 31) / 32) * L.ny * L.nz;
   const int rows = warps >= 16LL * num_sms ? 8 : 1;
   const int parts = warps <= 2LL * num_sms ? 7 : (warps <= 6LL * num_sms ? 3 : 1);
