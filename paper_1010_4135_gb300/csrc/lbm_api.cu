@@ -325,10 +325,12 @@ int auto_zchunk(const Layout& L, int num_sms) {
 // figures (200 x 4 x 4 one plane, 3.7 us against 7.3 with four; 96^3 12
 // planes, exactly 288 units, 29.6 against 37.2 with four).
 // r <= 80: as many long chunks per column as w waves of slots hold, w =
-// ceil(r / 45), each 0.95 r / w planes as far as that number allows, and the
-// rest of the column in 4-plane chunks that fill the slots left (128^3: 26 + 4,
-// 59.9 us, 12 + 8 68.9, one more long chunk per column, 24 + 4, 79.7;
-// 192 x 128 x 128: 36 + 4, 82.8 against 89.5).
+// ceil(r / 45), each 0.85 r / w planes as far as that number allows, and the
+// rest of the column in 4-plane chunks that fill the slots left (128^3: 25 + 4,
+// 60.0 us, 12 + 8 68.9, one more long chunk per column, 24 + 4, 79.7;
+// 192 x 128 x 128: 34 + 4, 82.7 against 89.5).  The share 0.85, against 0.95,
+// 0.9, 0.8 and 0.75, over 47 grids of r = 11 to 80: in all 1.5 % less than 0.95,
+// most where the columns are many and short (300 x 80 x 80 59.9 us against 64.7).
 // Beyond, 32 planes ending in 8-plane chunks: the re-read planes at the chunks'
 // ends count more than the last wave (256^3 383 us, the best of 60 379).
 lbm::ZSched auto_zsched(const Layout& L, int num_sms, const lbm::PairShape& shape) {
@@ -341,7 +343,7 @@ lbm::ZSched auto_zsched(const Layout& L, int num_sms, const lbm::PairShape& shap
     const int nl = (int)((long long)w * slots / tiles);
     if (nl >= 1 && L.nz > 4) {
       const int lo = (L.nz - 4) / (nl + 1) + 1, hi = (L.nz - 4) / nl;
-      int zc = (int)std::lround(0.95 * r / w);
+      int zc = (int)std::lround(0.85 * r / w);
       if (zc > hi) zc = hi;
       if (zc < lo) zc = lo;
       return lbm::make_zsched(L.nz, zc, 4);
