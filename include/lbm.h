@@ -174,8 +174,13 @@ LBM_API int lbm_set_wait_limit(lbm_sim* sim, uint32_t polls);
  * step's health flag reports it. */
 LBM_API int lbm_init(lbm_sim* sim, const double* rho, const double* u, const double* T, int32_t on_device);
 
-/* Advance n >= 0 time steps: per step one boundary-fill kernel and one fused
- * step kernel on the sim's stream; returns without waiting. */
+/* Advance n >= 0 time steps: per step one fused step kernel on the sim's
+ * stream, after a boundary-fill kernel where the step does not take care of
+ * the boundary layers itself (see the variants above; the FP64 step wraps
+ * periodic axes as it reads and leaves the other faces to the fill).  The
+ * kernels are chained (programmatic dependent launch): each starts while the
+ * one before it ends, and touches memory only after it has completed.
+ * Returns without waiting. */
 LBM_API int lbm_step(lbm_sim* sim, int64_t n);
 
 /* (rho, u, T) of every interior cell in double precision (relations e1-e3,
@@ -293,7 +298,7 @@ LBM_API int64_t lbm_steps_done(const lbm_sim* sim);
 /* Advance n sims by `steps` time steps together.  Per step, one launch of the
  * persistent FP32 tile kernel walks a descriptor table holding every grid's
  * tiles (uneven grids, different constants and boundaries are fine), plus a
- * fill launch only for boundary layers that kernel does not write itself.
+ * fill launch only for boundary layers that kernel does not handle itself.
  * All sims must be FP32 with the default tiled variant and the same scheme,
  * live on the current device and share one stream (sims[0]'s); 1 <= n <=
  * LBM_MAX_BATCH.  Each sim's result is bitwise the one lbm_step gives it

@@ -2,7 +2,7 @@
 //
 // A CTA owns a TX x TY column of cells and marches it through a chunk of z
 // planes.  Each plane of all 15 fields, with a two-cell halo in x and y, is
-// brought into shared memory by one 4D TMA copy (box 36 x 12 x 1 x 15) into a
+// brought into shared memory by one 4D TMA copy (box 40 x 12 x 1 x 15) into a
 // ring of NSLOT slots; completion is tracked by one mbarrier per slot, and the
 // copy for plane z+NSLOT is issued as soon as plane z is retired, so a full
 // step of compute hides each copy.  Per cell the kernel forms the moments,

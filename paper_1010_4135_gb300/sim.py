@@ -105,7 +105,8 @@ class Sim:
 
     def set_launch(self, variant="tiled", zchunk: int = 0, ztail: int = 0):
         """FP32 step kernel: "tiled" (32 x 8 TMA plane tiles, cell pairs, boundary layers
-        handled by the step; default), "tiled64" and "split" (the same kernel), "tiled_fill" (periodic layers by a fill launch), "tiled_single" (one cell per thread) or "plain";
+        handled by the step; default), "tiled64" and "split" (the same kernel), "tiled_fill"
+        (periodic layers by a fill launch), "tiled_single" (one cell per thread) or "plain";
         zchunk = z planes per CTA (0 = auto); ztail > 0 (pair kernels): the end of each
         tile column is split into short chunks of ztail planes, launched last."""
         v = {"tiled": A.LBM_VARIANT_TILED, "plain": A.LBM_VARIANT_PLAIN,
