@@ -319,11 +319,15 @@ int auto_zchunk(const Layout& L, int num_sms) {
 
 // Chunks of the pair kernel when none are set, from the planes per CTA slot
 // (two slots per SM), r = tiles nz / slots.
-// r < 12: equal chunks.  A unit takes its planes and about 1.5 planes' time
-// to start; a plane takes about 1.45 us on an SM with one unit and 1.95 us
-// where two share it.  The chunk with the least time for all waves by these
-// figures (200 x 4 x 4 one plane, 3.7 us against 7.3 with four; 96^3 12
-// planes, exactly 288 units, 29.6 against 37.2 with four).
+// r < 12: chunks as even as they go (two lengths, one plane apart), as many as
+// take the least time over all waves by these figures: a unit takes its planes
+// and about 1.5 planes' time to start; a plane takes about 1.45 us on an SM
+// with one unit and 1.95 us where two share it, where units of both lengths
+// meet.  Even chunks against chunks of one length and a remainder (us per
+// step): 64^3, 7 of 4 planes and 12 of 3 per column, exactly 304 units, 10.2
+// against 11.4 with 16 of 4; 500 x 40 x 44 33.4 against 36.3; 200 x 4 x 4 one
+// plane, 3.7 us against 7.3 with four; 96^3 8 of 12, 288 units, 29.6 against
+// 37.2 with four-plane ones; 110 grids, none slower by more than 1 %.
 // r <= 80: as many long chunks per column as w waves of slots hold, w =
 // ceil(r / 45), each 0.85 r / w planes as far as that number allows, and the
 // rest of the column in 4-plane chunks that fill the slots left (128^3: 25 + 4,
@@ -352,16 +356,18 @@ lbm::ZSched auto_zsched(const Layout& L, int num_sms, const lbm::PairShape& shap
   }
   int best = 1;
   double least = 0.0;
-  for (int zc = 1; zc <= L.nz && zc <= 24; ++zc) {
-    const double planes = zc + 1.5;
-    const long long units = tiles * ((L.nz + zc - 1) / zc), rem = units % slots;
-    const double t = (units / slots) * planes * 1.95 + (rem == 0 ? 0.0 : planes * (rem <= num_sms ? 1.45 : 1.95));
-    if (zc == 1 || t < least) {
+  for (int n = 1; n <= L.nz && tiles * (n - 1) < 2 * slots; ++n) {  // more than two waves only add starts
+    const int longest = (L.nz + n - 1) / n;
+    const double planes = 0.5 * (longest + (double)L.nz / n) + 1.5;
+    const long long units = tiles * n, rem = units % slots;
+    const double t = (units / slots) * planes * 1.95 +
+                     (rem == 0 ? 0.0 : (rem <= num_sms ? (longest + 1.5) * 1.45 : planes * 1.95));
+    if (n == 1 || t < least) {
       least = t;
-      best = zc;
+      best = n;
     }
   }
-  return lbm::make_zsched(L.nz, best, 0);
+  return lbm::even_zsched(L.nz, best);
 }
 
 unsigned step_faces(const lbm_sim* s) {
@@ -629,9 +635,11 @@ int run_steps(lbm_sim* s, int64_t n) {
     if (rc) return rc;
   }
   const bool pair = s->prec == LBM_FP32 && pair_variant(s->variant);
-  const lbm::PairShape shape = lbm::pair_shape();
   unsigned written = 0, own = 0;
   const lbm::WtDesc wt = write_through(s, &written, &own);
+  const lbm::ZSched zs = !pair           ? lbm::ZSched()
+                         : s->zchunk > 0 ? lbm::make_zsched(s->L.nz, s->zchunk, s->ztail)
+                                         : auto_zsched(s->L, s->num_sms, lbm::pair_shape());
   for (int64_t k = 0; k < n; ++k) {
     void* fin = s->fbuf[s->cur];
     void* fout = s->fbuf[s->cur ^ 1];
@@ -642,8 +650,6 @@ int run_steps(lbm_sim* s, int64_t n) {
       LBM_LAUNCH(s, LBM_KERNEL_FILL, lbm::launch_fill(s->prec, fin, s->L, s->md, s->mf, s->bc, mask, s->st));
     if (s->prec == LBM_FP32 && s->variant != LBM_VARIANT_PLAIN) {
       if (pair) {
-        const lbm::ZSched zs = s->zchunk > 0 ? lbm::make_zsched(s->L.nz, s->zchunk, s->ztail)
-                                             : auto_zsched(s->L, s->num_sms, shape);
         LBM_LAUNCH(s, LBM_KERNEL_STEP,
                    lbm::launch_step_pair(s->scheme, s->tmap[s->cur], (const float*)fin, (float*)fout, s->L, s->mf, wt,
                                          s->rd, zs, s->flags, s->wait_limit, s->st));

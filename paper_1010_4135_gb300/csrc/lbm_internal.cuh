@@ -293,6 +293,16 @@ inline ZSched make_zsched(int nz, int zc, int zt) {
   return z;
 }
 
+// nch chunks (1 <= nch <= nz) as even as they go, the long ones first
+inline ZSched even_zsched(int nz, int nch) {
+  ZSched z;
+  z.zc = (nz + nch - 1) / nch;
+  z.zt = z.zc > 1 ? z.zc - 1 : 1;
+  z.nch = nch;
+  z.nbig = z.zc > 1 ? nz - nch * (z.zc - 1) : nch;
+  return z;
+}
+
 cudaError_t launch_step_pair(int scheme, const CUtensorMap& map, const float* fin, float* fout, const Layout& L,
                              const Model<float>& m, const WtDesc& wt, const RecoverDesc& rd,
                              const ZSched& zs, unsigned* flags, unsigned wait_limit, cudaStream_t st);
