@@ -413,7 +413,8 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS_PER_SM)
 }
 
 // Persistent batched step: two CTAs per SM take the units of every grid in
-// the descriptor table (grid-major, then z chunk, then tile; each unit one
+// the descriptor table (the long chunks of all grids, then the short ones;
+// grid-major, then z chunk, then tile; each unit one
 // z-march of a TX x TY column of one grid) from a work queue, one atomic
 // increment per unit, so fast and slow CTAs balance.  Every CTA overshoots
 // the queue once; the last CTA to finish resets the queue for the next
@@ -440,11 +441,12 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS_PER_SM)
     __syncthreads();
     if (u >= tab.total_units || timed_out) break;
     int e = 0;
-    while (e + 1 < tab.n && u >= tab.item[e + 1].first_unit) ++e;
+    const bool late = u >= tab.long_units;
+    while (e + 1 < tab.n && u >= (late ? tab.item[e + 1].first_short : tab.item[e + 1].first_long)) ++e;
     const BatchItem& it = tab.item[e];
-    const long long local = u - it.first_unit;
+    const long long local = u - (late ? it.first_short : it.first_long);
     const long long per_chunk = (long long)it.tiles_x * it.tiles_y;
-    const int chunk = (int)(local / per_chunk);
+    const int chunk = (int)(local / per_chunk) + (late ? it.zs.nbig : 0);
     const int t = (int)(local % per_chunk);
     // the unit's descriptors as locals: read through the runtime index e, the
     // table's constants would otherwise be re-loaded at every use in the plane

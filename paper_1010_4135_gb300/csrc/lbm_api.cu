@@ -675,16 +675,53 @@ int run_steps(lbm_sim* s, int64_t n) {
 }
 
 // Chunks of the batched kernel for sims with none set, from the planes per CTA
-// slot over all grids, r: units come from one queue, so only the last ones
-// leave slots idle, and about 1.7 sqrt(r) planes balance that against the time
-// a unit takes to start (us per step: two 64^3 grids, r = 7, 4 planes 29.1, 8
-// 30.5, 24 64.7; eight 64^3, r = 27, 8 + 0 89.4, 24 109; four grids of 64^3 to
-// 192 x 128 x 128, r = 82, 14 + 8 193, 24 202; eight 128^3, r = 216, 28 463, 16
-// 471; with 512 x 256 x 256, r = 647, 32 1231, 24 1247, 16 1283).
-lbm::ZSched batch_zsched(int nz, double r) {
-  int zc = (int)std::lround(1.7 * std::sqrt(r));
-  zc = zc < 2 ? 2 : (zc > 32 ? 32 : zc);
-  return lbm::make_zsched(nz, zc, zc >= 10 && zc <= 20 ? 8 : 0);
+// slot over all grids, r.  The long chunks of all grids are taken from the
+// queue before any short one, so that the SMs run out of work together (us per
+// step, the short ones of each grid after its long ones before, now):
+// r < 12: chunks as even as they go, the shortest whose units fit the slots at
+// once (two 64^3 25.0, 22.3; three 37.0, 30.8; six 200 x 4 x 4 8.6, 8.0).
+// r < 70: w = ceil(r / 35) waves of long chunks of 0.85 r / w planes, or as
+// many more as it takes for them to be w waves, and 4-plane ones (four 64^3
+// 48.3, 40.8; eight 78.8, 72.5; two 128^3 123.7, 116.1).
+// r < 400: 28 planes, then 4 or 8 (four grids of 64^3 to 192 x 128 x 128, r = 82,
+// 174.7, 168.4; thirty 64^3 249, 240; eight 128^3 437, 422).
+// Beyond, 32 planes and no short ones: the units' starts and re-read planes
+// count more than the last wave (512 x 256 x 256 and eight 128^3, r = 647, 1167
+// us; 28 + 4 1172, 40 + 8 1166).
+struct BatchChunk {
+  int zc, zt;  // zt < 0: even chunks of at most zc planes
+  lbm::ZSched of(int nz) const { return zt < 0 ? lbm::even_zsched(nz, (nz + zc - 1) / zc) : lbm::make_zsched(nz, zc, zt); }
+};
+BatchChunk batch_chunk(lbm_sim* const* sims, int n, const lbm::PairShape& shape, int slots) {
+  long long tiles[lbm::kMaxBatch], all = 0;
+  double r = 0.0;
+  for (int i = 0; i < n; ++i) {
+    const Layout& L = sims[i]->L;
+    tiles[i] = (long long)((L.nx + shape.tx - 1) / shape.tx) * ((L.ny + shape.ty - 1) / shape.ty);
+    all += tiles[i];
+    r += (double)tiles[i] * L.nz / slots;
+  }
+  if (r < 12.0) {
+    if (all > slots) {
+      const int zc = (int)std::lround(1.7 * std::sqrt(r));
+      return {zc < 2 ? 2 : zc, 0};
+    }
+    for (int zc = 1;; ++zc) {  // ends: a chunk per column is a unit per tile
+      long long units = 0;
+      for (int i = 0; i < n; ++i) units += tiles[i] * ((sims[i]->L.nz + zc - 1) / zc);
+      if (units <= slots) return {zc, -1};
+    }
+  }
+  if (r >= 400.0) return {32, 0};
+  if (r >= 70.0) return {28, r < 110.0 ? 4 : 8};
+  const int w = (int)std::ceil(r / 35.0);
+  int zc = (int)std::lround(0.85 * r / w);
+  for (; zc < r / w; ++zc) {
+    long long units = 0;
+    for (int i = 0; i < n; ++i) units += tiles[i] * (sims[i]->L.nz > 4 ? (sims[i]->L.nz - 4) / zc : 0);
+    if (units <= (long long)w * slots) break;
+  }
+  return {zc, 4};
 }
 
 int batch_check(lbm_sim* const* sims, int32_t n) {
@@ -714,12 +751,8 @@ int run_batch(lbm_sim* const* sims, int32_t n, int64_t steps) {
   thread_local static lbm::BatchTable tab;  // built on the host, passed by value to the kernel
   unsigned written[lbm::kMaxBatch], own[lbm::kMaxBatch];
   lbm::WtDesc wt[lbm::kMaxBatch];
-  double planes = 0.0;  // tile planes of all grids
-  for (int i = 0; i < n; ++i) {
-    const Layout& L = sims[i]->L;
-    wt[i] = write_through(sims[i], &written[i], &own[i]);
-    planes += (double)((L.nx + shape.tx - 1) / shape.tx) * ((L.ny + shape.ty - 1) / shape.ty) * L.nz;
-  }
+  for (int i = 0; i < n; ++i) wt[i] = write_through(sims[i], &written[i], &own[i]);
+  const BatchChunk chunk = batch_chunk(sims, n, shape, shape.ctas_per_sm * s0->num_sms);
   for (int64_t k = 0; k < steps; ++k) {
     long long units = 0;
     for (int i = 0; i < n; ++i) {
@@ -741,9 +774,15 @@ int run_batch(lbm_sim* const* sims, int32_t n, int64_t steps) {
       it.tiles_x = (s->L.nx + shape.tx - 1) / shape.tx;
       it.tiles_y = (s->L.ny + shape.ty - 1) / shape.ty;
       it.zs = s->zchunk > 0 ? lbm::make_zsched(s->L.nz, s->zchunk, s->ztail)
-                            : batch_zsched(s->L.nz, planes / ((double)shape.ctas_per_sm * s0->num_sms));
-      it.first_unit = units;
-      units += (long long)it.tiles_x * it.tiles_y * it.zs.nch;
+                            : chunk.of(s->L.nz);
+      it.first_long = units;
+      units += (long long)it.tiles_x * it.tiles_y * it.zs.nbig;
+    }
+    tab.long_units = units;
+    for (int i = 0; i < n; ++i) {
+      lbm::BatchItem& it = tab.item[i];
+      it.first_short = units;
+      units += (long long)it.tiles_x * it.tiles_y * (it.zs.nch - it.zs.nbig);
     }
     tab.n = n;
     tab.wait_limit = s0->wait_limit;

@@ -308,8 +308,9 @@ cudaError_t launch_step_pair(int scheme, const CUtensorMap& map, const float* fi
                              const ZSched& zs, unsigned* flags, unsigned wait_limit, cudaStream_t st);
 
 // Descriptor table of a batched step (passed by value as the kernel
-// parameter): one entry per grid, units [first_unit, first_unit +
-// tiles_x * tiles_y * zs.nch) in z-chunk-major order.
+// parameter): one entry per grid, units [first_long, first_long + tiles_x *
+// tiles_y * zs.nbig) for its long chunks and [first_short, ...) for the others,
+// in z-chunk-major order.
 constexpr int kMaxBatch = 48;
 struct BatchItem {
   const float* fin;
@@ -321,14 +322,14 @@ struct BatchItem {
   RecoverDesc rd;
   ZSched zs;
   int tiles_x, tiles_y;
-  long long first_unit;
+  long long first_long, first_short;  // first unit of its long, of its short chunks
 };
 struct BatchTable {
   CUtensorMap map[kMaxBatch];
   BatchItem item[kMaxBatch];
   int n;
   unsigned wait_limit;
-  long long total_units;
+  long long long_units, total_units;  // the long chunks of all grids come first
   unsigned long long* queue;  // next unit to take (0 at launch; reset by the last CTA)
   unsigned* done;             // CTAs finished (0 at launch; reset by the last CTA)
 };
