@@ -5,7 +5,7 @@
 // one sum are aligned to the largest exponent among them, E: v = n 2^(E -
 // 1079), |n| < 2^57, which holds all 53 bits of values down to 2^-4 of the
 // largest (floats: all 24 bits down to 2^-33) and truncates smaller ones below
-// 2^-56 of it.  Any combination of the values whose coefficients' magnitudes
+// 2^-56 of it (the moments' sums: two bits more).  Any combination of the values whose coefficients' magnitudes
 // sum to less than 64 is exact, and is rounded once, to 53 bits, when it
 // becomes a double; a double evaluation rounds at each operation, at 2^-53 of
 // its operands.  Sums whose largest exponent is outside [EMIN, EMAX]
@@ -19,8 +19,13 @@ namespace lbm {
 namespace fx {
 
 constexpr int EMIN = 200, EMAX = 1900;
-constexpr int SHIFT = 4;                   // 53-bit mantissas, top bit at bit 56
-constexpr int BIAS = 1023 + 52 + SHIFT;    // n counts units of 2^(E - BIAS)
+// S: 53-bit mantissas' top bit at bit 52 + S; n counts units of 2^(E - bias(S)).
+// Sums of coefficients below 64 use SHIFT, plain sums of a cell's 15 values
+// MOMENT_SHIFT, which truncates four times less (FP64 moments of 82 thousand
+// noisy cells against quad precision, relative 2-norm of u: SHIFT 9.0e-16,
+// MOMENT_SHIFT 2.1e-16, double sums 5.3e-16).
+constexpr int SHIFT = 4, MOMENT_SHIFT = 6;
+constexpr int bias(int S) { return 1023 + 52 + S; }
 
 // Magnitude pattern of a value (of a double its high word), which orders like
 // the magnitudes' exponents, and the double-biased exponent E of the largest.
@@ -42,29 +47,32 @@ __device__ __forceinline__ long long aligned(unsigned long long n, unsigned sh, 
   return ((long long)n ^ s) - s;
 }
 
-// v in units of 2^(E - BIAS), truncated toward zero; E is in range and at
+// v in units of 2^(E - bias(S)), truncated toward zero; E is in range and at
 // least v's exponent (zeros and subnormals are shifted out).
+template <int S = SHIFT>
 __device__ __forceinline__ long long to_fixed(double v, int E) {
   const int h = __double2hiint(v);
   const unsigned l = (unsigned)__double2loint(v);
-  const unsigned long long n = (((unsigned long long)(((unsigned)h & 0xfffffu) | 0x100000u) << 32) | l) << SHIFT;
+  const unsigned long long n = (((unsigned long long)(((unsigned)h & 0xfffffu) | 0x100000u) << 32) | l) << S;
   return aligned(n, (unsigned)(E - (mag(v) >> 20)), h);
 }
+template <int S = SHIFT>
 __device__ __forceinline__ long long to_fixed(float v, int E) {
   const int b = __float_as_int(v);
-  const unsigned long long n = (unsigned long long)(((unsigned)b & 0x7fffffu) | 0x800000u) << (SHIFT + 29);
+  const unsigned long long n = (unsigned long long)(((unsigned)b & 0x7fffffu) | 0x800000u) << (S + 29);
   return aligned(n, (unsigned)(E - (1023 - 127) - (mag(v) >> 23)), b);
 }
 
-// n 2^(E - BIAS), rounded to 53 bits (a tie away from zero).
+// n 2^(E - bias(S)), rounded to 53 bits (a tie away from zero).
+template <int S = SHIFT>
 __device__ __forceinline__ double from_fixed(long long n, int E) {
   const long long s = n >> 63;
   unsigned long long a = (unsigned long long)((n ^ s) - s);
   const int lz = __clzll((long long)a);
   a = a << (lz & 63);
-  // top bit 63 - lz: biased exponent E - BIAS + 1023 + 63 - lz, less one for
+  // top bit 63 - lz: biased exponent E - bias(S) + 1023 + 63 - lz, less one for
   // the mantissa's leading bit, which the sum below adds to it
-  const unsigned e = (unsigned)(E - BIAS + 1023 + 62 - lz);
+  const unsigned e = (unsigned)(E - bias(S) + 1023 + 62 - lz);
   const unsigned long long q = (a >> 11) + ((a >> 10) & 1ull);  // a carry to 2^53 raises the exponent
   const unsigned hi = ((unsigned)(q >> 32) + (e << 20)) | ((unsigned)(s >> 32) & 0x80000000u);
   return a == 0 ? 0.0 : __hiloint2double((int)hi, (int)(unsigned)q);
@@ -88,17 +96,18 @@ __device__ __forceinline__ void moments_fixed(const Model<double>& m, const R f[
   }
   long long n[NV];
 #pragma unroll
-  for (int i = 0; i < NV; ++i) n[i] = to_fixed(f[i], E);
+  for (int i = 0; i < NV; ++i) n[i] = to_fixed<MOMENT_SHIFT>(f[i], E);
   const long long sa = ((n[1] + n[2]) + (n[3] + n[4])) + (n[5] + n[6]);
   const long long pp = n[7] + n[8], pm = n[9] + n[10], mp = n[11] + n[12], mm = n[13] + n[14];
   const long long sd = (pp + pm) + (mp + mm);
   const long long dz = ((n[7] + n[9]) + (n[11] + n[13])) - ((n[8] + n[10]) + (n[12] + n[14]));
-  rho = from_fixed(n[0] + sa + sd, E);
-  const double px = fma(m.c1, from_fixed(n[1] - n[2], E), m.s * from_fixed((pp + pm) - (mp + mm), E));
-  const double py = fma(m.c1, from_fixed(n[3] - n[4], E), m.s * from_fixed((pp + mp) - (pm + mm), E));
-  const double pz = fma(m.c1, from_fixed(n[5] - n[6], E), m.s * from_fixed(dz, E));
-  const double f0 = sizeof(R) == 8 ? (double)f[0] : from_fixed(n[0], E);
-  const double en = fma(m.eta0sq, f0, fma(m.c1sq, from_fixed(sa, E), m.c2sq * from_fixed(sd, E)));
+  auto sum = [&](long long a) { return from_fixed<MOMENT_SHIFT>(a, E); };
+  rho = sum(n[0] + sa + sd);
+  const double px = fma(m.c1, sum(n[1] - n[2]), m.s * sum((pp + pm) - (mp + mm)));
+  const double py = fma(m.c1, sum(n[3] - n[4]), m.s * sum((pp + mp) - (pm + mm)));
+  const double pz = fma(m.c1, sum(n[5] - n[6]), m.s * sum(dz));
+  const double f0 = sizeof(R) == 8 ? (double)f[0] : sum(n[0]);
+  const double en = fma(m.eta0sq, f0, fma(m.c1sq, sum(sa), m.c2sq * sum(sd)));
   const double ir = 1.0 / rho;
   ux = px * ir;
   uy = py * ir;
