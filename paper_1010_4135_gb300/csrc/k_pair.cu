@@ -98,7 +98,7 @@ struct Opt {
 // using the same barriers; jb advances by the unit's plane count.  All
 // threads of the CTA call it together; timed_out is uniform.
 template <int SCHEME, class G, class O>
-__device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* __restrict__ fin,
+__device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* fin,
                                           float* __restrict__ fout, const Layout& L, const Model<float>& m,
                                           const WtDesc& wt, const RecoverDesc& rd, int x0, int y0, int z0,
                                           int nzc,
@@ -393,7 +393,7 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* _
 
 template <int SCHEME, class G, class O>
 __global__ void __launch_bounds__(G::THREADS, G::CTAS_PER_SM)
-    step_pair_kernel(const __grid_constant__ CUtensorMap tin, const float* __restrict__ fin, float* __restrict__ fout,
+    step_pair_kernel(const __grid_constant__ CUtensorMap tin, const float* fin, float* __restrict__ fout,
                      Layout L, Model<float> m, WtDesc wt, RecoverDesc rd, ZSched zs, unsigned* __restrict__ flags,
                      unsigned wait_limit) {
   extern __shared__ __align__(128) unsigned char smem[];

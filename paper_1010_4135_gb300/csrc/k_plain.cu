@@ -117,21 +117,21 @@ __device__ __noinline__ double conv2_double(double c, double x0, double x1, doub
 struct Nb {
   unsigned k[4];
 };
-__device__ __forceinline__ double at(const double* __restrict__ f, unsigned k) { return __ldg(f + k); }
+__device__ __forceinline__ double at(const double* f, unsigned k) { return f[k]; }
 
 // The values a velocity's update reads besides the cell's own, upwind to
 // downwind m2, m1, p1 along each axis of a diagonal velocity; for an axis one
 // m2, m1, p1 along its axis and the four lateral neighbours.  R..: reversed
 // axes (negative components).
 template <bool RX, bool RY, bool RZ>
-__device__ __forceinline__ void diag_load(const double* __restrict__ f, const Nb& X, const Nb& Y, const Nb& Z,
+__device__ __forceinline__ void diag_load(const double* f, const Nb& X, const Nb& Y, const Nb& Z,
                                           double v[9]) {
   v[0] = at(f, X.k[RX ? 3 : 0]); v[1] = at(f, X.k[RX ? 2 : 1]); v[2] = at(f, X.k[RX ? 1 : 2]);
   v[3] = at(f, Y.k[RY ? 3 : 0]); v[4] = at(f, Y.k[RY ? 2 : 1]); v[5] = at(f, Y.k[RY ? 1 : 2]);
   v[6] = at(f, Z.k[RZ ? 3 : 0]); v[7] = at(f, Z.k[RZ ? 2 : 1]); v[8] = at(f, Z.k[RZ ? 1 : 2]);
 }
 template <bool R>
-__device__ __forceinline__ void axis_load(const double* __restrict__ f, const Nb& A, const Nb& B, const Nb& C,
+__device__ __forceinline__ void axis_load(const double* f, const Nb& A, const Nb& B, const Nb& C,
                                           double v[9]) {
   v[0] = at(f, A.k[R ? 3 : 0]); v[1] = at(f, A.k[R ? 2 : 1]); v[2] = at(f, A.k[R ? 1 : 2]);
   v[3] = at(f, B.k[1]); v[4] = at(f, B.k[2]); v[5] = at(f, C.k[1]); v[6] = at(f, C.k[2]);
@@ -227,7 +227,7 @@ __device__ __forceinline__ Nb neighbours(int i, int n, bool periodic, unsigned k
 // itself.  kax, kdg: factors of axis_sum and diag_conv2.
 template <int SCHEME, bool R1>
 __global__ void __launch_bounds__(256, 3)
-    step_fp64_kernel(const double* __restrict__ fin, double* __restrict__ fout, Layout L, Model<double> m, double kax,
+    step_fp64_kernel(const double* fin, double* __restrict__ fout, Layout L, Model<double> m, double kax,
                      double kdg, unsigned per, int parts, unsigned* __restrict__ flags) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = (blockIdx.y / parts) * blockDim.y + threadIdx.y;
@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(256, 3)
 // -> 5.9).
 template <int SCHEME, bool R1>
 __global__ void __launch_bounds__(32)
-    step_fp64_pairs_kernel(const double* __restrict__ fin, double* __restrict__ fout, Layout L, Model<double> m,
+    step_fp64_pairs_kernel(const double* fin, double* __restrict__ fout, Layout L, Model<double> m,
                            double kax, double kdg, unsigned per, unsigned* __restrict__ flags) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y / 7, z = blockIdx.z, part = blockIdx.y % 7;

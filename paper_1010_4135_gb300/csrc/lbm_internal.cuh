@@ -105,7 +105,11 @@ struct WtDesc {
 // called chain_start() (or ended), so the launch latency (2 to 4 us between
 // small dependent kernels) overlaps that kernel's end.  Such a kernel touches
 // no memory that other kernels use before chain_wait(), which waits until every
-// kernel before it has completed and its writes are visible.
+// kernel before it has completed and its writes are visible to ordinary loads.
+// Such a kernel is resident while its predecessor still writes, so what it
+// reads is not read-only for its lifetime: no __ldg and no `const T*
+// __restrict__` parameter (the non-coherent path) on memory that another kernel
+// writes.
 __device__ __forceinline__ void chain_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
