@@ -85,8 +85,11 @@ using pm::ld2;
 // FULL: every tile lies inside the grid (nx and ny multiples of the tile), so
 // the activity tests fold away.  R1: dt = tau (dt/tau = 1, keep_2 = 0).  RD:
 // FP64 temperature recovery.  XF, WALL: layers of extrapolating / reflecting
-// x faces, of reflecting y and z faces, formed as they are read.  FEW: fewer
-// than four rows and periodic y, so a row has several images.
+// x faces, of reflecting y and z faces, formed as they are read.  FEW: some
+// grid has fewer than four rows and periodic y, so its rows have several images
+// (the others' rows keep their one address; found by walking a grid's rows, the
+// images cost every grid of the launch: 256^3 with dt = tau/2 3468 us, now 427,
+// beside 200 x 3 x 3 in a batch 3496, now 414).
 template <bool FULL_, bool R1_, bool RD_, bool XF_, bool WALL_, bool FEW_>
 struct Opt {
   static constexpr bool FULL = FULL_, R1 = R1_, RD = RD_, XF = XF_, WALL = WALL_, FEW = FEW_;
@@ -213,10 +216,11 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* f
   // (E/rho - u^2)/b, -inf or NaN when u^2 is inf or NaN.
   float2 hmin_rho = make_float2(INFINITY, INFINITY), hmin_T = hmin_rho, hsum = make_float2(0.f, 0.f);
   // periodic images of this pair (element offsets from its own index, 0 = none):
-  // one per axis, or with fewer than four rows (FEW) several y ones
+  // one per axis, or several y ones in a grid of fewer than four rows (few)
   unsigned img_y = 0, img_x = 0;
+  const bool few = O::FEW && wt.per[1] && L.ny < 4;
   if (act0) {
-    if (!O::FEW && wt.per[1]) img_y = (unsigned)L.sx * (unsigned)(y < 2 ? L.ny : (y >= L.ny - 2 ? -L.ny : 0));
+    if (!few && wt.per[1]) img_y = (unsigned)L.sx * (unsigned)(y < 2 ? L.ny : (y >= L.ny - 2 ? -L.ny : 0));
     if (wt.per[0]) img_x = (unsigned)(x == 0 ? L.nx : (x == L.nx - 2 ? -L.nx : 0));
   }
   // store the pair's new values of plane k, the deferred fields (late) or the others, and their images
@@ -240,11 +244,12 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* f
       if (img_y) put(g + img_y);
       if (img_x) put(g + img_x);
     }
-    if (O::FEW && wt.per[1] && act0) {
+    if (few && act0) {
 #pragma unroll 1
-      for (int q = -2; q < L.ny + 2; ++q)
-        if (q < 0 || q >= L.ny)
-          if ((q - y) % L.ny == 0) put(g + (unsigned)(q - y) * (unsigned)L.sx);
+      for (int j = 0; j < 4; ++j) {  // the four layers: -2, -1, ny, ny + 1
+        const int q = j < 2 ? j - 2 : L.ny + j - 2;
+        if ((q - y) % L.ny == 0) put(g + (unsigned)(q - y) * (unsigned)L.sx);
+      }
     }
   };
   // faces whose layers are formed here, from the moments of the cells at the
