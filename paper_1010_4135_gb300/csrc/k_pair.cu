@@ -490,18 +490,30 @@ struct Need {
 };
 
 // The forms that exist: NND with dt = tau and no recovery (every run of the
-// paper) has one per boundary need, everything else one form with all parts.
+// paper) has one per boundary need; NND with another relaxation time or with
+// recovery has one for whole and one for cut tiles, each with x faces (256^3,
+// us per step against the form with all parts: dt = tau/2 387, 427; recovery
+// 459, 505); everything else (the upwind schemes, 368 and 375; walls or few
+// rows with either of those; both walls and few rows) one form with all parts.
 using FullPlain = Opt<true, true, false, false, false, false>;
 using FullFaces = Opt<true, true, false, true, false, false>;
 using Plain = Opt<false, true, false, false, false, false>;
 using Faces = Opt<false, true, false, true, false, false>;
 using Walls = Opt<false, true, false, true, true, false>;
 using FewRows = Opt<false, true, false, true, false, true>;
+using FullRelax = Opt<true, false, false, true, false, false>;
+using Relax = Opt<false, false, false, true, false, false>;
+using FullRecover = Opt<true, false, true, true, false, false>;
+using Recover = Opt<false, false, true, true, false, false>;
 using General = Opt<false, false, true, true, true, true>;
 
 template <int SCHEME, class F>
 void with_form(const Need& n, F f) {
   if constexpr (SCHEME == LBM_SCHEME_NND) {
+    if (!n.few && !n.wall && (n.rd || !n.r1)) {
+      if (n.rd) return n.full ? f(FullRecover()) : f(Recover());
+      return n.full ? f(FullRelax()) : f(Relax());
+    }
     if (n.r1 && !n.rd && !(n.few && n.wall)) {
       if (n.few) return f(FewRows());
       if (n.wall) return f(Walls());
@@ -546,7 +558,8 @@ void launch_batch_scheme(const BatchTable& tab, int grid, cudaStream_t st) {
 }  // namespace
 
 cudaError_t prepare_pair_kernels() {
-  cudaError_t e = set_attributes<LBM_SCHEME_NND, FullPlain, FullFaces, Plain, Faces, Walls, FewRows, General>();
+  cudaError_t e = set_attributes<LBM_SCHEME_NND, FullPlain, FullFaces, Plain, Faces, Walls, FewRows, FullRelax, Relax,
+                                 FullRecover, Recover, General>();
   if (e == cudaSuccess) e = set_attributes<LBM_SCHEME_UPWIND2, General>();
   if (e == cudaSuccess) e = set_attributes<LBM_SCHEME_UPWIND1, General>();
   return e;
