@@ -84,8 +84,8 @@ enum { LBM_HEALTH_NONFINITE = 1u, LBM_HEALTH_RHO = 2u, LBM_HEALTH_T = 4u, LBM_HE
  * two x-adjacent cells per thread in packed f32x2 arithmetic (default); the
  * step kernel takes care of periodic axes, reflecting faces and extrapolating
  * x faces itself, so no fill launch is needed between steps (but for odd nx at
- * the x-hi face, odd ny at a reflecting y-hi face, extrapolating y and z faces
- * and FP64 temperature recovery); TILED_FILL = the TILED kernel with the
+ * the x-hi face, odd ny at a reflecting y-hi face and extrapolating y and z
+ * faces); TILED_FILL = the TILED kernel with the
  * periodic layers left to a fill launch before each step; TILED_SINGLE = 32 x
  * 8 tiles, one cell per thread; PLAIN = one thread per cell reading global
  * memory; TILED64 and TILED_SPLIT (once 64 x 8 tiles, and two warp groups per

@@ -176,7 +176,7 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* f
     float2 v[NV];
 #pragma unroll
     for (int i = 0; i < NV; ++i) v[i] = z0 == 0 ? ld2(P0 + i * PL + c) : h1[i];
-    const pm::Mom r = pm::moments<O::RD>(m, rd, v, P0, c, PL, act0, act1);
+    const pm::Mom r = pm::moments<false>(m, rd, v, P0, c, PL, act0, act1);
     const pm::Mom e1 = pm::wall_layer<2>(r, false), e2 = pm::wall_layer<2>(r, true);
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
@@ -277,6 +277,9 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* f
     // moments (relations e1-e3), health, equilibrium and the per-field update
     const pm::Mom r = pm::moments<O::RD>(m, rd, F, P0, c, PL, act0, act1);
     {
+      // the layers take the FP32 moments, as the fill forms them, also where
+      // the cell's own were recovered in FP64
+      auto face_moments = [&]() { return O::RD && rd.on ? pm::moments<false>(m, rd, F, P0, c, PL, act0, act1) : r; };
       // layers beyond the faces this pair touches: into the plane tile's halo
       // (x: read by this thread only; y: by the row above or below too, a row
       // of this warp), or in place of the plane above
@@ -285,7 +288,7 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* f
         for (int lo = 0; lo < 2; ++lo) {
           if (!(lo ? at_xlo : at_xhi)) continue;
           float* t = const_cast<float*>(P0) + c + (lo ? -2 : 2);
-          const pm::Mom e = pm::x_layers(r, lo ? wt.xlo : wt.xhi, lo);
+          const pm::Mom e = pm::x_layers(face_moments(), lo ? wt.xlo : wt.xhi, lo);
 #pragma unroll
           for (int i = 0; i < NV; ++i) *reinterpret_cast<float2*>(t + i * PL) = pm::feq(m, e, i);
         }
@@ -296,7 +299,7 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* f
           for (int q = 0; q < 4; ++q) {  // lo inner, lo outer, hi inner, hi outer
             if (!(q < 2 ? at_ylo : at_yhi)) continue;
             float* t = const_cast<float*>(P0) + c + (q < 2 ? -1 - q : q - 1) * BX;
-            const pm::Mom e = pm::wall_layer<1>(r, q & 1);
+            const pm::Mom e = pm::wall_layer<1>(face_moments(), q & 1);
 #pragma unroll
             for (int i = 0; i < NV; ++i) *reinterpret_cast<float2*>(t + i * PL) = pm::feq(m, e, i);
           }
@@ -304,7 +307,7 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* f
         __syncwarp();
       }
       if (wt.zhi && z0 + k == L.nz - 1) {
-        const pm::Mom e = pm::wall_layer<2>(r, false);
+        const pm::Mom e = pm::wall_layer<2>(face_moments(), false);
 #pragma unroll
         for (int i = 0; i < NV; ++i) Z1[i] = pm::feq(m, e, i);
       }
@@ -360,7 +363,7 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* f
       float2 v[NV];
 #pragma unroll
       for (int i = 0; i < NV; ++i) v[i] = ld2(P0 + i * PL + c);
-      const pm::Mom e = pm::wall_layer<2>(pm::moments<O::RD>(m, rd, v, P0, c, PL, act0, act1), over == 1);
+      const pm::Mom e = pm::wall_layer<2>(pm::moments<false>(m, rd, v, P0, c, PL, act0, act1), over == 1);
 #pragma unroll
       for (int i = 0; i < NV; ++i)
         if (pm::deferred<SCHEME>(i)) top[i] = pm::feq(m, e, i);
@@ -493,7 +496,7 @@ struct Need {
 // paper) has one per boundary need; NND with another relaxation time or with
 // recovery has one for whole and one for cut tiles, each with x faces (256^3,
 // us per step against the form with all parts: dt = tau/2 387, 427; recovery
-// 459, 505); everything else (the upwind schemes, 368 and 375; walls or few
+// 398, 505); everything else (the upwind schemes, 368 and 375; walls or few
 // rows with either of those; both walls and few rows) one form with all parts.
 using FullPlain = Opt<true, true, false, false, false, false>;
 using FullFaces = Opt<true, true, false, true, false, false>;
