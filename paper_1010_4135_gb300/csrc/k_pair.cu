@@ -306,6 +306,9 @@ __device__ __forceinline__ void pair_unit(const CUtensorMap* tin, const float* f
         }
         __syncwarp();
       }
+      // in every form, although only WALL ones can take it: compiled out of
+      // the others it makes them slower (us: 256^3, 150 steps, 59942, without
+      // 60169; 128^3, 150 steps, 9358, 9406; four served grids 17919, 18105)
       if (wt.zhi && z0 + k == L.nz - 1) {
         const pm::Mom e = pm::wall_layer<2>(face_moments(), false);
 #pragma unroll
