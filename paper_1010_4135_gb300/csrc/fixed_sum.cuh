@@ -63,6 +63,17 @@ __device__ __forceinline__ long long to_fixed(float v, int E) {
   return aligned(n, (unsigned)(E - (1023 - 127) - (mag(v) >> 23)), b);
 }
 
+// The same for a value that a limiter compares and does not add: its exponent
+// may be above E, and from 2^(E + 4) on it saturates at [2^59, 2^60) units, more
+// than twice any difference of two values of exponents up to E.
+__device__ __forceinline__ long long to_fixed_limiter(double v, int E) {
+  constexpr int UP = 3;
+  const int h = __double2hiint(v);
+  const unsigned l = (unsigned)__double2loint(v);
+  const unsigned long long n = (((unsigned long long)(((unsigned)h & 0xfffffu) | 0x100000u) << 32) | l) << (SHIFT + UP);
+  return aligned(n, (unsigned)max(E + UP - (mag(v) >> 20), 0), h);
+}
+
 // n 2^(E - bias(S)), rounded to 53 bits (a tie away from zero).
 template <int S = SHIFT>
 __device__ __forceinline__ double from_fixed(long long n, int E) {

@@ -89,6 +89,7 @@ using fx::from_fixed;
 using fx::in_range;
 using fx::mag;
 using fx::to_fixed;
+using fx::to_fixed_limiter;
 
 __device__ __forceinline__ long long clamp64(long long x, long long lo, long long hi) { return min(max(x, lo), hi); }
 
@@ -137,19 +138,34 @@ __device__ __forceinline__ void axis_load(const double* f, const Nb& A, const Nb
   v[3] = at(f, B.k[1]); v[4] = at(f, B.k[2]); v[5] = at(f, C.k[1]); v[6] = at(f, C.k[2]);
 }
 
+// The values that are added set the scale of a stencil.  m2 and p1 only bound
+// the limited differences (NND), or do not enter (p1 of the upwind schemes, m2
+// of the first-order one), so a large one costs the others no bits: with them
+// in the scale, a neighbour K times the rest left the convection sum a relative
+// error of K 2^-56.  UPWIND2 adds m2.
+template <int SCHEME>
+constexpr bool kAddsM2 = SCHEME == LBM_SCHEME_UPWIND2;
+template <int SCHEME>
+__device__ __forceinline__ long long fixed_m2(double v, int E) {
+  return kAddsM2<SCHEME> ? to_fixed(v, E) : to_fixed_limiter(v, E);
+}
+
 // Twice the convection sum of a diagonal velocity.
 template <int SCHEME>
 __device__ __forceinline__ double diag_conv2(double c, const double v[9]) {
   int mx = mag(c);
 #pragma unroll
-  for (int j = 0; j < 9; ++j) mx = max(mx, mag(v[j]));
+  for (int a = 0; a < 3; ++a) {
+    mx = max(mx, mag(v[3 * a + 1]));
+    if (kAddsM2<SCHEME>) mx = max(mx, mag(v[3 * a]));
+  }
   const int E = mx >> 20;
   if (!in_range(E)) return conv2_double<SCHEME>(c, v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7], v[8]);
   const long long n = to_fixed(c, E);
   long long s = 0;
 #pragma unroll
   for (int a = 0; a < 3; ++a)
-    s += grad2<SCHEME>(to_fixed(v[3 * a], E), to_fixed(v[3 * a + 1], E), n, to_fixed(v[3 * a + 2], E));
+    s += grad2<SCHEME>(fixed_m2<SCHEME>(v[3 * a], E), to_fixed(v[3 * a + 1], E), n, to_fixed_limiter(v[3 * a + 2], E));
   return from_fixed(s, E);
 }
 
@@ -159,16 +175,19 @@ __device__ __forceinline__ double diag_conv2(double c, const double v[9]) {
 // Laplacian, or twice the convection alone when the term is off.
 template <int SCHEME>
 __device__ __forceinline__ double axis_sum(double c, const double v[9], bool dissipation) {
-  int mx = mag(c);
+  int mx = max(mag(c), mag(v[1]));
+  if (kAddsM2<SCHEME>) mx = max(mx, mag(v[0]));
+  if (dissipation) {
 #pragma unroll
-  for (int j = 0; j < 7; ++j) mx = max(mx, mag(v[j]));
+    for (int j = 2; j < 7; ++j) mx = max(mx, mag(v[j]));
+  }
   const int E = mx >> 20;
   if (!in_range(E)) {
     const double conv2 = 2.0 * grad_pos<SCHEME>(v[0], v[1], c, v[2]);
     return dissipation ? 5.0 * conv2 - (((v[1] + v[2]) + (v[3] + v[4])) + (v[5] + v[6]) - 6.0 * c) : conv2;
   }
-  const long long n = to_fixed(c, E), n1 = to_fixed(v[1], E), n2 = to_fixed(v[2], E);
-  long long s = grad2<SCHEME>(to_fixed(v[0], E), n1, n, n2);
+  const long long n = to_fixed(c, E), n1 = to_fixed(v[1], E), n2 = to_fixed_limiter(v[2], E);
+  long long s = grad2<SCHEME>(fixed_m2<SCHEME>(v[0], E), n1, n, n2);
   if (dissipation) {
     s = 5 * s + 6 * n - (n1 + n2);
 #pragma unroll
