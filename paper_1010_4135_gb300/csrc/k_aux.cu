@@ -277,19 +277,31 @@ template <typename R, int N>
 struct FieldAcc;
 template <int N>
 struct FieldAcc<double, N> {
-  double s[N];
-  int largest = 0;
+  // the two values of a load, then up to FOLD such sums, then those: a lane's
+  // chain of additions, and its rounding where all values are alike, does not
+  // grow with the grid (256^3, uniform values, 432 of them per lane, relative
+  // error of the total, 400 values: rms 5.9e-15, worst 1.2e-14 in one chain;
+  // 5.6e-16, 1.5e-15 so)
+  static constexpr int FOLD = 32;
+  double s[N], total[N];
+  int largest = 0, loads = 0;
   __device__ FieldAcc() {
 #pragma unroll
-    for (int i = 0; i < N; ++i) s[i] = 0.0;
+    for (int i = 0; i < N; ++i) s[i] = total[i] = 0.0;
   }
   __device__ __forceinline__ void add(int i, const double v[2]) {
-    s[i] += v[0];
-    s[i] += v[1];
+    s[i] += v[0] + v[1];
     largest = max(largest, max(fx::mag(v[0]), fx::mag(v[1])));
   }
-  __device__ __forceinline__ void renorm() {}
-  __device__ __forceinline__ double value(int i) const { return s[i]; }
+  __device__ __forceinline__ void renorm() {
+    if (++loads % FOLD != 0) return;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      total[i] += s[i];
+      s[i] = 0.0;
+    }
+  }
+  __device__ __forceinline__ double value(int i) const { return total[i] + s[i]; }
   // a NaN or infinity has a high word above every finite one
   __device__ __forceinline__ bool bad() const { return !(__hiloint2double(largest, 0) < 1e300); }
 };
