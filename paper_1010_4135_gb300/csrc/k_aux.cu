@@ -302,6 +302,7 @@ struct FieldAcc<double, N> {
     }
   }
   __device__ __forceinline__ double value(int i) const { return total[i] + s[i]; }
+  __device__ __forceinline__ bool in_range() const { return true; }
   // a NaN or infinity has a high word above every finite one
   __device__ __forceinline__ bool bad() const { return !(__hiloint2double(largest, 0) < 1e300); }
 };
@@ -320,12 +321,8 @@ struct FieldAcc<float, N> {
     for (int i = 0; i < N; ++i) s[i].renorm();
   }
   __device__ __forceinline__ double value(int i) const { return s[i].value(); }
-  __device__ __forceinline__ bool bad() const {
-    bool nan = false;
-#pragma unroll
-    for (int i = 0; i < N; ++i) nan = nan || isnan(s[i].hi.x + s[i].lo.x) || isnan(s[i].hi.y + s[i].lo.y);
-    return nan || !(largest < 3.0e38f);
-  }
+  __device__ __forceinline__ bool in_range() const { return !(largest >= 1e30f); }  // 2^27 such values stay finite
+  __device__ __forceinline__ bool bad() const { return !(largest < 3.0e38f); }
 };
 
 // 16-byte vector loads of float / double rows (read once: streaming hint).
@@ -369,31 +366,53 @@ __global__ void __launch_bounds__(RED_THREADS) conserved_kernel(const R* __restr
   const int nr = gridDim.x * RED_ROWS;
   constexpr int VW = 16 / (int)sizeof(R);  // elements per 16-byte load
   const R* fg = f + (long long)grp * RED_GF * L.fs;
-  for (int r = blockIdx.x * RED_ROWS + slot; r < nrows; r += nr) {
-    // interior rows start at x = OX (a multiple of 8 elements): 16-byte aligned
-    const R* row = fg + L.at(0, r % L.ny, r / L.ny);
-    for (int x0 = lane * VW; x0 < L.nx; x0 += 32 * VW) {
-      // the last vector may reach up to VW - 1 elements past the row end,
-      // into the row's halo and padding (inside the buffer); masked below
-      R v[RED_GF][VW];
+  auto each = [&](auto take) {  // every vector of this lane, masked past the row end
+    for (int r = blockIdx.x * RED_ROWS + slot; r < nrows; r += nr) {
+      // interior rows start at x = OX (a multiple of 8 elements): 16-byte aligned
+      const R* row = fg + L.at(0, r % L.ny, r / L.ny);
+      for (int x0 = lane * VW; x0 < L.nx; x0 += 32 * VW) {
+        // the last vector may reach up to VW - 1 elements past the row end,
+        // into the row's halo and padding (inside the buffer); masked below
+        R v[RED_GF][VW];
 #pragma unroll
-      for (int i = 0; i < RED_GF; ++i) load16(row + i * L.fs + x0, v[i]);
-      if (x0 + VW > L.nx) {
+        for (int i = 0; i < RED_GF; ++i) load16(row + i * L.fs + x0, v[i]);
+        if (x0 + VW > L.nx) {
 #pragma unroll
-        for (int i = 0; i < RED_GF; ++i)
+          for (int i = 0; i < RED_GF; ++i)
 #pragma unroll
-          for (int k = 0; k < VW; ++k)
-            if (x0 + k >= L.nx) v[i][k] = R(0);
+            for (int k = 0; k < VW; ++k)
+              if (x0 + k >= L.nx) v[i][k] = R(0);
+        }
+        take(v);
       }
-#pragma unroll
-      for (int i = 0; i < RED_GF; ++i) acc.add(i, v[i]);
-      acc.renorm();
     }
+  };
+  each([&](const R(&v)[RED_GF][VW]) {
+#pragma unroll
+    for (int i = 0; i < RED_GF; ++i) acc.add(i, v[i]);
+    acc.renorm();
+  });
+  double sums[RED_GF];
+#pragma unroll
+  for (int i = 0; i < RED_GF; ++i) sums[i] = acc.value(i);
+  if (!acc.in_range()) {
+    // float sums of such values may have left the float range: once more in double
+#pragma unroll
+    for (int i = 0; i < RED_GF; ++i) sums[i] = 0.0;
+    each([&](const R(&v)[RED_GF][VW]) {
+#pragma unroll
+      for (int k = 0; k < VW; ++k)
+#pragma unroll
+        for (int i = 0; i < RED_GF; ++i) sums[i] += (double)v[i][k];
+    });
   }
-  if (acc.bad()) atomicOr(flags, (unsigned)LBM_HEALTH_NONFINITE);
+  bool bad = acc.bad();
+#pragma unroll
+  for (int i = 0; i < RED_GF; ++i) bad = bad || fx::mag(sums[i]) > 0x7ff00000;  // a NaN, on the integer ALUs
+  if (bad) atomicOr(flags, (unsigned)LBM_HEALTH_NONFINITE);
 #pragma unroll
   for (int i = 0; i < RED_GF; ++i) {
-    double v = acc.value(i);
+    double v = sums[i];
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
     if (lane == 0) wsum[warp][grp * RED_GF + i] = v;
