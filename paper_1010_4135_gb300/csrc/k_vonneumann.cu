@@ -88,6 +88,11 @@ struct Mat {
     for (int o = VT / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
     return v;
   }
+  __device__ int max(int v) const {
+#pragma unroll
+    for (int o = VT / 2; o > 0; o >>= 1) v = ::max(v, __shfl_xor_sync(mask, v, o));
+    return v;
+  }
   __device__ double max(double v) const {
 #pragma unroll
     for (int o = VT / 2; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(mask, v, o));
@@ -176,7 +181,7 @@ __device__ void build_g(const Mat& M, const double* st, const double* p, const d
 }
 
 // Spectral radius of M (destroyed), or +inf if the QR iteration does not
-// converge; the same value in every lane.  rot: VN rotations of the group.
+// converge or M is not finite; the same value in every lane.  rot: VN rotations of the group.
 struct Rot {
   cd s;
   double c;
@@ -185,6 +190,19 @@ template <class Mat>
 __device__ double spectral_radius(const Mat& M, Rot* rot) {
   constexpr int VT = Mat::VT;
   const int n = VN, g = M.g;
+  // Entries far from 1 are scaled by a power of two (exact): the products of
+  // four entries below (two squared norms) then stay in range.
+  int largest = 0;  // high word of the largest component
+  for (int r = g; r < n; r += VT)
+    for (int c = 0; c < n; ++c)
+      largest = max(largest, max(__double2hiint(M.at(r, c).re) & 0x7fffffff, __double2hiint(M.at(r, c).im) & 0x7fffffff));
+  const int e2 = (M.max(largest) >> 20) - 1023;
+  const int scale = e2 < 1024 && (e2 > 64 || e2 < -64) ? e2 : 0;
+  if (scale != 0) {
+    for (int r = g; r < n; r += VT)
+      for (int c = 0; c < n; ++c) M.at(r, c) = mk(scalbn(M.at(r, c).re, -scale), scalbn(M.at(r, c).im, -scale));
+    M.sync();
+  }
   // Householder reduction to upper Hessenberg form (similarity, eigenvalues kept)
 #pragma unroll 1
   for (int k = 0; k + 2 < n; ++k) {
@@ -226,6 +244,7 @@ __device__ double spectral_radius(const Mat& M, Rot* rot) {
   // size anyway, and without the norm floor a cluster of tiny eigenvalues
   // (those of G for dt = tau are O(Courant number)) is never split off
   const double ulp = 2.220446049250313e-16;
+  const double TINY = 1e-220;  // |x| = 1e-110 beside a norm of 2^-64 at least
   double nrm = 0.0;
   for (int r = g; r < n; r += VT)
     for (int c = r > 0 ? r - 1 : 0; c < n; ++c) nrm = fmax(nrm, cabs1(M.at(r, c)));
@@ -281,11 +300,12 @@ __device__ double spectral_radius(const Mat& M, Rot* rot) {
       const double px = norm2(x), pn = px + norm2(y);
       double cg = 1.0;
       cd sg = mk(0.0, 0.0);
-      if (px >= 1e-280) {
+      // |y| is above ulp times the matrix' norm, so px pn is a normal number
+      if (px >= TINY) {
         const double rs = rsqrt(px * pn);  // 1 / (|x| |(x, y)|)
         cg = px * rs;
         sg = rs * (x * cconj(y));
-      } else if (pn >= 1e-280) {  // x = 0 beside y: exchange the rows
+      } else if (pn >= TINY) {  // x is nothing beside y: exchange the rows
         cg = 0.0;
         sg = mk(1.0, 0.0);
       }
@@ -313,7 +333,7 @@ __device__ double spectral_radius(const Mat& M, Rot* rot) {
     for (int j = l + g; j <= hi; j += VT) M.at(j, j) = M.at(j, j) + mu;
     M.sync();
   }
-  return radius;
+  return scalbn(radius, scale);
 }
 
 // Item t of the batch: parameter set t / per_param, then state, direction and
