@@ -374,6 +374,10 @@ cudaError_t launch_vn_max_growth(const double* states, int nstates, const double
                                  cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(out, 0, sizeof(double) * nparams, st);
   if (e != cudaSuccess) return e;
+  int device = 0, num_sms = 0;
+  e = cudaGetDevice(&device);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, device);
+  if (e != cudaSuccess) return e;
   // Lanes per matrix: with fewer than 16 matrices per SM four lanes leave too
   // few warps to cover the FP64 pipe's latency, with more eight repeat too much
   // scalar work (us: 1920 matrices 1448 with four, 1031 with eight; 5760
@@ -384,7 +388,7 @@ cudaError_t launch_vn_max_growth(const double* states, int nstates, const double
                                                                         dissipation,
                                                                         reinterpret_cast<unsigned long long*>(out));
   };
-  if (items < 16LL * 152) run(vn_kernel<8>, VN_THREADS / 8);
+  if (items < 16LL * num_sms) run(vn_kernel<8>, VN_THREADS / 8);
   else run(vn_kernel<4>, VN_THREADS / 4);
   return cudaGetLastError();
 }
