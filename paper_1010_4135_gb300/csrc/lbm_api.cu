@@ -683,11 +683,14 @@ int run_steps(lbm_sim* s, int64_t n) {
 // r < 70: w = ceil(r / 35) waves of long chunks of 0.85 r / w planes, or as
 // many more as it takes for them to be w waves, and 4-plane ones (four 64^3
 // 48.3, 40.8; eight 78.8, 72.5; two 128^3 123.7, 116.1).
-// r < 400: 28 planes, then 4 or 8 (four grids of 64^3 to 192 x 128 x 128, r = 82,
-// 174.7, 168.4; thirty 64^3 249, 240; eight 128^3 437, 422).
+// r < 400: 28 planes, then 8 (four grids of 64^3 to 192 x 128 x 128, r = 82,
+// 174.7 before, 169.2; thirty 64^3 249, 240; eight 128^3 437, 421).  Against 28 + 4:
+// 17 batches of r = 70 to 110 0.5 % less in all (-2 .. +2.4 %), eight of r = 216 to
+// 364 1.0 % less (-2.5 .. +0.9 %); against 32 and no short ones, less in each of 11.
 // Beyond, 32 planes and no short ones: the units' starts and re-read planes
-// count more than the last wave (512 x 256 x 256 and eight 128^3, r = 647, 1167
-// us; 28 + 4 1172, 40 + 8 1166).
+// count more than the last wave (us, 28 + 8 against 32: r = 431, three batches,
+// 760 762, 796 798, 775 767; r = 647, 1183 1168, 1147 1134; 28 + 4 754, 794, 765,
+// 1173, 1127: no less for the longest, 512 x 256 x 256 and eight 128^3).
 struct BatchChunk {
   int zc, zt;  // zt < 0: even chunks of at most zc planes
   lbm::ZSched of(int nz) const { return zt < 0 ? lbm::even_zsched(nz, (nz + zc - 1) / zc) : lbm::make_zsched(nz, zc, zt); }
@@ -713,7 +716,7 @@ BatchChunk batch_chunk(lbm_sim* const* sims, int n, const lbm::PairShape& shape,
     }
   }
   if (r >= 400.0) return {32, 0};
-  if (r >= 70.0) return {28, r < 110.0 ? 4 : 8};
+  if (r >= 70.0) return {28, 8};
   const int w = (int)std::ceil(r / 35.0);
   int zc = (int)std::lround(0.85 * r / w);
   for (; zc < r / w; ++zc) {
