@@ -15,19 +15,23 @@ measurements.  The best choice depends on the grid's shape and the SM count,
 so it is measured: each candidate runs a few steps of the sim's own state on a
 scratch copy of the sim (its own workspace, so the user's state and step count
 are untouched), timed with CUDA events on the scratch sim's stream; the choice
-is applied and cached per (device, grid, precision, scheme, boundary kinds) in
-a JSON file (LBM_TUNE_CACHE, default
+is applied and cached per (device, grid, precision, scheme, boundary kinds,
+candidates, kernel form and sources) in a JSON file (LBM_TUNE_CACHE, default
 ~/.cache/paper_1010_4135_gb300/launch.json), so each shape is tuned once.
 FP64 sims always use the plain kernel and are not tuned.
 """
 from __future__ import annotations
 
+import functools
+import glob
+import hashlib
 import json
 import os
 import threading
 
 import torch
 
+CSRC = os.path.join(os.path.dirname(os.path.abspath(__file__)), "csrc")
 ZCHUNKS = (0, 1, 2, 4, 6, 8, 12, 14, 16, 20, 24, 28, 32, 40, 48)  # 0: the library's own choice
 ZTAILS = (0, 8, 16)  # 0: equal chunks; a tail length is tried only below the chunk length
 VARIANTS = ("tiled", "tiled64")
@@ -77,6 +81,27 @@ def key_of(sims, batched: bool, device_name: str | None = None, sms: int | None 
     return "|".join(parts)
 
 
+@functools.lru_cache(maxsize=None)
+def kernel_hash() -> str:
+    """Hash of the library's sources: a measurement is of one version of the kernels."""
+    h = hashlib.sha256()
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cuh"))):
+        h.update(os.path.basename(path).encode())
+        with open(path, "rb") as fh:
+            h.update(fh.read())
+    return h.hexdigest()[:16]
+
+
+def entry_of(sims, batched: bool, zchunks=ZCHUNKS, variants=None, device_name: str | None = None,
+             sms: int | None = None) -> str:
+    """Name of a cache entry: key_of, the z chunks measured, the kernels'
+    version, and what else a sim's kernel form goes by (dt = tau, recovery)."""
+    forms = [("dt=tau" if s.config["dt"] == s.config["tau"] else "dt!=tau") + (":recovery" if s.t_recovery else "")
+             for s in sims]
+    return "|".join([key_of(sims, batched, device_name, sms, variants), "chunks" + ",".join(str(int(z)) for z in zchunks),
+                     ",".join(forms), kernel_hash()])
+
+
 def _time(run, steps: int, warmup: int) -> float:
     run(warmup)
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -107,6 +132,7 @@ def measure(sims, zchunks=ZCHUNKS, steps: int = 10, warmup: int = 2, batched: bo
                 s.get_f(out=f)
                 s.sync()
                 c = s.clone(stream=torch.cuda.current_stream(s.device))
+                c.set_t_recovery(s.t_recovery)
                 scratch.append((c, f))
 
             def ms(launch):
@@ -163,7 +189,7 @@ def _tune(sims, zchunks, steps, use_cache, path, batched, key=None, variants=VAR
     if any(s.config["precision"] not in ("fp32", 1) for s in sims):
         return {"variant": None, "zchunk": None, "ztail": None, "ms": None, "cached": False, "timings": {}}
     path = path or cache_path()
-    key = key or key_of(sims, batched, variants=variants)
+    key = key or entry_of(sims, batched, zchunks, variants)
     hit = _load(path).get(key) if use_cache else None
     if hit is not None:
         for s in sims:

@@ -38,6 +38,7 @@ class Sim:
                             precision=precision, bc_lo=bc_lo, bc_hi=bc_hi, fixed_lo=fixed_lo, fixed_hi=fixed_hi,
                             scheme=scheme, dissipation=dissipation, device=device)
         self.launch = ("tiled", 0, 0)  # (variant, zchunk, ztail)
+        self.t_recovery = 0.0  # set_t_recovery
         self.shape = (int(nz), int(ny), int(nx))
         self.prec = PRECISIONS[precision] if isinstance(precision, str) else int(precision)
         self.dtype = np.float64 if self.prec == A.LBM_FP64 else np.float32
