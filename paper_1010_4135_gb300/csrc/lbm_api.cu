@@ -685,8 +685,8 @@ int run_steps(lbm_sim* s, int64_t n) {
 // 48.3, 40.8; eight 78.8, 72.5; two 128^3 123.7, 116.1).
 // r < 400: 28 planes, then 8 (four grids of 64^3 to 192 x 128 x 128, r = 82,
 // 174.7 before, 169.2; thirty 64^3 249, 240; eight 128^3 437, 421).  Against 28 + 4:
-// 17 batches of r = 70 to 110 0.5 % less in all (-2 .. +2.4 %), eight of r = 216 to
-// 364 1.0 % less (-2.5 .. +0.9 %); against 32 and no short ones, less in each of 11.
+// 17 batches of r = 70 to 110 0.5 % less in all (-2 .. +2.4 %), 14 of r = 216 to
+// 364 0.3 % less (-2.5 .. +1.2 %); against 32 and no short ones, less in each of 11.
 // Beyond, 32 planes and no short ones: the units' starts and re-read planes
 // count more than the last wave (us, 28 + 8 against 32: r = 431, three batches,
 // 760 762, 796 798, 775 767; r = 647, 1183 1168, 1147 1134; 28 + 4 754, 794, 765,
