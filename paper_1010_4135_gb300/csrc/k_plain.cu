@@ -75,12 +75,12 @@ __global__ void __launch_bounds__(256) step_plain_kernel(const float* __restrict
 // FP32 or integer ones, so the step is bound by the FP64 operations it needs
 // and everything linear in f is taken off that pipe: the moments' sums, the
 // convection's differences, minmods and sums, and the Laplacian, run in 64-bit
-// fixed point (fixed_sum.cuh; the values aligned are a velocity's stencil, or
-// a cell's 15 values).  The largest sum, five times twice the convection of an
+// fixed point (fixed_sum.cuh; the values aligned are those of a velocity's
+// stencil, or of one of a cell's sums).  The largest sum, five times twice the convection of an
 // axis velocity (|difference| <= 2, |minmod| <= |difference|) less its
 // Laplacian, is at most 52 times the largest value (a diagonal velocity's
-// convection 24 times).  256^3: 13.3 -> 4.3 ms per step (417 -> 112 FP64
-// operations per cell; the FP64 pipe 84 -> 69 % busy, the integer ALUs 74 %:
+// convection 24 times).  256^3: 13.3 -> 4.2 ms per step (417 -> 112 FP64
+// operations per cell; the FP64 pipe 84 -> 72 % busy, the integer ALUs 74 %:
 // both near their rates); 300 x 80 x 80 with walls 1.68 -> 0.57 ms.
 // Aligning by one multiplication where the values are within 2^4 of each other
 // saves 900 of 3400 ALU instructions, but the cells at shocks and zero
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(256, 3)
 // issued before the moments' arithmetic: on a grid of a few hundred rows the
 // step is one warp's latency, and the stencils' loads after the moments were a
 // second trip to the L2 (150 x 1 x 1: 5.2 -> 4.3 us per step, 200 x 4 x 4: 6.3
-// -> 5.9).
+// -> 5.9, with a scale per sum of the moments 6.0).
 template <int SCHEME, bool R1>
 __global__ void __launch_bounds__(32)
     step_fp64_pairs_kernel(const double* fin, double* __restrict__ fout, Layout L, Model<double> m,
