@@ -157,8 +157,8 @@ LBM_API int lbm_set_launch(lbm_sim* sim, int32_t variant, int32_t zchunk, int32_
  * then large and of opposite sign); its relative rounding error is about
  * 2^-24 kappa with kappa = 1 + (6 c1^2 |A_axis| + 8 c2^2 |A_diag| + u^2)/(b T).
  * Cells with kappa > kappa_max, or with T <= 0 in FP32, recompute rho, u and
- * T from their 15 values in FP64.  kappa_max = 0 turns it off; otherwise
- * kappa_max >= 1 (LBM_EINVAL else).  The paper has no counterpart: it fixes
+ * T from their 15 values in FP64; boundary layers take the FP32 moments.
+ * kappa_max = 0 turns it off; otherwise kappa_max >= 1 (LBM_EINVAL else).  The paper has no counterpart: it fixes
  * no precision. */
 LBM_API int lbm_set_t_recovery(lbm_sim* sim, double kappa_max);
 

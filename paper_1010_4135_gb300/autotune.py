@@ -98,8 +98,8 @@ def entry_of(sims, batched: bool, zchunks=ZCHUNKS, variants=None, device_name: s
     version, and what else a sim's kernel form goes by (dt = tau, recovery)."""
     forms = [("dt=tau" if s.config["dt"] == s.config["tau"] else "dt!=tau") + (":recovery" if s.t_recovery else "")
              for s in sims]
-    return "|".join([key_of(sims, batched, device_name, sms, variants), "chunks" + ",".join(str(int(z)) for z in zchunks),
-                     ",".join(forms), kernel_hash()])
+    chunks = "chunks" + ",".join(str(int(z)) for z in zchunks)
+    return "|".join([key_of(sims, batched, device_name, sms, variants), chunks, ",".join(forms), kernel_hash()])
 
 
 def _time(run, steps: int, warmup: int) -> float:

@@ -28,7 +28,8 @@ def test_residents_together_keep_the_automatic_launch(monkeypatch, tune):
         return real(sims, n)
 
     monkeypatch.setattr(serve.S, "step_batch", step_batch)
-    tr = workloads.serving_trace(seed=7, n=5, rate=200.0, grids=((16, 16, 16), (24, 16, 16), (32, 16, 8)), steps=(200, 600))
+    tr = workloads.serving_trace(seed=7, n=5, rate=200.0, grids=((16, 16, 16), (24, 16, 16), (32, 16, 8)),
+                                 steps=(6000, 12000))  # long enough that requests overlap
     srv = serve.Server(max_batch=3, tick=16, prep_workers=5, tune=tune)
     done = srv.run(tr)
     assert len(done) == 5 and all(j.health == 0 for j in done)
